@@ -214,13 +214,12 @@ hz_status hz_plan_create(hz_medium* med, const hz_solver_opts* opts, int max_nrh
 
 /* Autotuner (the paper has no counterpart; it tunes this implementation's
  * launch shapes).  Times candidate launch shapes of the kernels that dominate
- * a solve on the plan's own buffers with CUDA events on `stream`: blocks per
- * SM and vectors per block of the CGS2 dot kernel, blocks per SM of the CGS2
- * update, nodes per block and columns per thread of the last-axis symbol
- * pass, and whether the x-inverse pass accumulates the weighted sum as it
+ * a solve on the plan's own buffers with CUDA events on `stream`: nodes per
+ * block and columns per thread of the last-axis symbol pass, and whether the x-inverse pass accumulates the weighted sum as it
  * goes, transforms the planes in place and gathers the sum afterwards, or
- * transforms each (row, node) line on its own and adds it into the output.  The choice is stored
- * in the plan and cached per (grid, K, max_nrhs, restart, precision) for the
+ * transforms each (row, node) line on its own and adds it into the output.
+ * The CGS2 kernels have one shape: dots_bps, dots_vc and upd_bps are accepted
+ * and reported but choose nothing.  The choice is stored in the plan and cached per (grid, K, max_nrhs, restart, precision) for the
  * process; later plans with the same key reuse it without timing.
  * Synchronous; overwrites the plan's work arrays (call before solving). */
 typedef struct {

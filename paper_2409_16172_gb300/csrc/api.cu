@@ -290,19 +290,25 @@ extern "C" hz_status hz_plan_create(hz_medium* med, const hz_solver_opts* opts, 
   p->tmp = tmp;
   if ((st = ensure_planes(p, opts->precision)) != HZ_OK) return fail(st);
   if ((st = p->arena.alloc(&p->V, size_t(m + 1) * B * n)) != HZ_OK) return fail(st);
-  // Z: FGMRES basis (c64); the FP64 path keeps one c128 work vector per rhs
+  // Z: FGMRES basis (c64); the FP64 path, the unpreconditioned and the left
+  // form keep one c128 work vector per rhs
   void* Z = nullptr;
-  const size_t zlen = opts->precision == 1 ? size_t(m) * B * n * es : size_t(B) * n * 16;
+  size_t zlen = opts->precision == 1 ? size_t(m) * B * n * es : size_t(B) * n * 16;
+  if (opts->no_precond || opts->left) zlen = std::max(zlen, size_t(B) * n * 16);
   if ((st = p->arena.alloc(reinterpret_cast<char**>(&Z), zlen)) != HZ_OK) return fail(st);
   p->Z = Z;
   if ((st = p->arena.alloc(&p->u, size_t(B) * n)) != HZ_OK) return fail(st);
   if ((st = p->arena.alloc(&p->f, size_t(B) * n)) != HZ_OK) return fail(st);
-  // block partial sums: the stencil residual (one per block), the CGS2 dot
-  // partials (2 (j+1) nblk doubles per rhs with at most 4 x 152 blocks over
-  // the launch, 8 vectors per chunk) and the update norms (<= 8 x 152 blocks)
+  // one budget for the tile exponents of the basis and the block partial
+  // sums: the stencil residual (one double per block), the CGS2 dot partials
+  // (2 (j+1) doubles per block) and the norms (one double per block)
   const int nblk = std::max(stencil_blocks(n), krylov_blocks(n, 1, 1));
-  p->partial_len = size_t(B) * (m + 2) * std::max(nblk, 1024) * 2;
+  const size_t budget = size_t(B) * (m + 2) * std::max(nblk, 1024) * 2;
+  const size_t evlen = size_t(B) * m * ((n + HZ_FX_TILE - 1) / HZ_FX_TILE);
+  p->partial_len = std::max(budget - (evlen + 1) / 2,
+                            size_t(m + 2) * 2 * HZ_CGS_BLOCKS * std::min(B, 4));
   if ((st = p->arena.alloc(&p->partial, p->partial_len)) != HZ_OK) return fail(st);
+  if ((st = p->arena.alloc(&p->ev, evlen)) != HZ_OK) return fail(st);
   *out = p;
   return HZ_OK;
 }

@@ -1,0 +1,71 @@
+// Block fixed-point form of FP64 vectors, and exact products in it.
+//
+// sm_103a executes 2 FP64 lanes per clock and SM (every DADD, DMUL, DFMA and
+// conversion to or from double: 1.9 measured), but 62 lanes of IMAD.WIDE
+// (32 x 32 + 64 bits).  Sums of products over FP64 vectors are therefore made
+// in integers: a tile of FX_TILE consecutive points shares one binary
+// exponent E (the largest of its real and imaginary parts), a value is the
+// integer v = x 2^(FX_TOP + 1023 - E) rounded to nearest, |v| <= 2^54, held
+// as two signed limbs v = hi 2^28 + lo, |hi| <= 2^26, |lo| <= 2^27.  A value
+// within a factor 2 of the tile's largest keeps all 53 bits; a smaller one is
+// exact to 2^-54 of the tile's largest, half an ulp of that value.  The four
+// limb products are exact and are added exactly in 64 bits.
+#pragma once
+#include "hz_internal.h"
+
+namespace hz {
+
+constexpr int FX_TILE = HZ_FX_TILE;  // points that share one exponent
+constexpr int FX_TOP = 53;           // bit of the leading one of a value with exponent E
+
+__device__ __forceinline__ int fx_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ int fx_exp(double2 z) { return max(fx_exp(z.x), fx_exp(z.y)); }
+
+// x 2^(FX_TOP + 1023 - E) to the nearest integer, E >= exponent of x; integer
+// operations only.  Subnormals count as zero.
+__device__ __forceinline__ long long fx_from(double x, int E) {
+  const int hi = __double2hiint(x);
+  const int ex = (hi >> 20) & 0x7ff;
+  const int sh = E - ex;
+  const unsigned long long m =
+      (static_cast<unsigned long long>((hi & 0xfffff) | 0x100000) << 32) | unsigned(__double2loint(x));
+  const int s = 9 + sh;  // m << 10 has its leading one at bit 62
+  const unsigned long long v = ((m << 10) + (1ull << ((s - 1) & 63))) >> (s & 63);
+  const long long sg = hi >> 31;
+  return (ex == 0 || s > 63) ? 0ll : ((static_cast<long long>(v) ^ sg) - sg);
+}
+
+// limbs of v: low 28 bits with sign, and the rest
+__device__ __forceinline__ int fx_lo(long long v) { return int(unsigned(v) << 4) >> 4; }
+__device__ __forceinline__ int fx_hi(long long v) { return int((v + (1ll << 27)) >> 28); }
+
+// a complex value as (re hi, re lo, im hi, im lo)
+__device__ __forceinline__ int4 fx_pack(double2 z, int E) {
+  const long long a = fx_from(z.x, E), b = fx_from(z.y, E);
+  return make_int4(fx_hi(a), fx_lo(a), fx_hi(b), fx_lo(b));
+}
+
+__device__ __forceinline__ long long mad_w(int a, int b, long long c) {
+  return static_cast<long long>(a) * b + c;
+}
+
+// hh 2^56 + x 2^28 + ll in units of 2^(56 - SH), rounded to nearest
+template <int SH>
+__device__ __forceinline__ long long fx_sum(long long hh, long long x, long long ll) {
+  const long long y = x + ((ll + (1ll << 27)) >> 28);
+  return (hh << SH) + ((y + (1ll << (27 - SH))) >> (28 - SH));
+}
+// fx_to's k for fx_sum<SH> of products of values whose (biased) exponents add
+// up to E
+template <int SH>
+__device__ __forceinline__ int fx_unit(int E) { return E + 56 - SH - 2 * FX_TOP - 2 * 1023; }
+
+// t 2^k; a result below the normal range is zero
+__device__ __forceinline__ double fx_to(long long t, int k) {
+  const double d = static_cast<double>(t);
+  const int hi = __double2hiint(d);
+  const int e = ((hi >> 20) & 0x7ff) + k;
+  return (t == 0 || e <= 0) ? 0.0 : __hiloint2double(hi + (k << 20), __double2loint(d));
+}
+
+}  // namespace hz

@@ -119,7 +119,9 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
   const int B = p->max_nrhs;
   const int prec = p->opts.precision;
   const double tol = p->opts.tol;
-  const long ldb = B;  // basis vector i of rhs b at V + (i * B + b) * n
+  const long ldb = B;  // basis vector i of rhs b at slot i * B + b
+  const Basis Q{reinterpret_cast<int4*>(p->V), p->ev, ldb, n, (n + HZ_FX_TILE - 1) / HZ_FX_TILE};
+  double2* W = p->V + long(m) * ldb * n;  // the current vector in FP64 (slot m)
 
   HZ_TRY(check_device(med));
   HZ_TRY(solve_ws_create(p));
@@ -167,10 +169,10 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
   // Q_M f; residuals are measured after Q_M, relative to ||Q_M f||.
   const bool left = p->opts.left != 0 && p->opts.no_precond == 0;
   if (left) {
-    HZ_TRY(precond_apply(p, prec, f, nullptr, nrhs, p->V, 1, st, nullptr));
+    HZ_TRY(precond_apply(p, prec, f, nullptr, nrhs, W, 1, st, nullptr));
     {
       PhaseScope ps(st, PH_NORM, 16.0 * Bn, 4.0 * Bn, 2);
-      HZ_TRY(launch_norm2(p->V, n, n, nrhs, p->partial, nblk_n, ks.bnorm, st));
+      HZ_TRY(launch_norm2(W, n, n, nrhs, p->partial, nblk_n, ks.bnorm, st));
     }
     HZ_CUDA(cudaMemcpyAsync(bnorm.data(), ks.bnorm, nrhs * sizeof(double), cudaMemcpyDeviceToHost, st));
     HZ_CUDA(cudaStreamSynchronize(st));
@@ -239,17 +241,17 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
   }
 
   for (;;) {
-    // true FP64 residual r = f - P u into V_0
+    // true FP64 residual r = f - P u
     {
       PhaseScope ps(st, PH_RESID, 64.0 * Bn + (med->a ? 8.0 * Bn : 0.0), 30.0 * Bn, 2);
-      HZ_TRY(launch_residual(med, u, f, p->V, n, nrhs, nullptr, p->partial, st));
+      HZ_TRY(launch_residual(med, u, f, W, n, nrhs, nullptr, p->partial, st));
       HZ_TRY(launch_reduce_r(p->partial, nblk_r, nrhs, w.rnorm2, st));
     }
     if (left) {
       // r <- Q_M r in place, and its norm
-      HZ_TRY(precond_apply(p, prec, p->V, nullptr, nrhs, p->V, 1, st, nullptr));
+      HZ_TRY(precond_apply(p, prec, W, nullptr, nrhs, W, 1, st, nullptr));
       PhaseScope ps(st, PH_NORM, 16.0 * Bn, 4.0 * Bn, 2);
-      HZ_TRY(launch_norm2(p->V, n, n, nrhs, p->partial, nblk_n, w.rnorm2, st));
+      HZ_TRY(launch_norm2(W, n, n, nrhs, p->partial, nblk_n, w.rnorm2, st));
     }
     HZ_CUDA(cudaMemcpyAsync(rn2.data(), w.rnorm2, nrhs * sizeof(double), cudaMemcpyDeviceToHost, st));
     HZ_CUDA(cudaStreamSynchronize(st));
@@ -293,14 +295,16 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
     HZ_CUDA(cudaMemcpyAsync(ks.n_active, &live, sizeof(int), cudaMemcpyHostToDevice, st));
     HZ_CUDA(cudaStreamSynchronize(st));  // host vectors above are reused next cycle
 
+    {
+      PhaseScope ps(st, PH_UPDATE, 32.0 * Bn, 0.0);
+      HZ_TRY(launch_encode(Q, W, n, 0, nrhs, ks.active, st));  // V_0 = r
+    }
     int maxit_left = 0;
     for (int b = 0; b < nrhs; ++b)
       if (!done[b]) maxit_left = std::max(maxit_left, p->opts.maxit - iters[b]);
     const int jmax = std::min(m, maxit_left);
     // one Arnoldi step for every live right-hand side (no host interaction)
     auto step = [&](int j, cudaStream_t st) -> hz_status {
-      const double2* Vj = p->V + long(j) * ldb * n;
-      double2* Vn = p->V + long(j + 1) * ldb * n;
       const double* sig_j = ks.sigma + long(j) * B;
       const double stb = Bn * ((prec == 1 ? 8.0 : 16.0) + 32.0 + (med->a ? 8.0 : 0.0));
       const double stf = Bn * (med->dim == 3 ? 30.0 : 26.0);
@@ -309,41 +313,47 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
         double2* zt = static_cast<double2*>(p->Z);
         {
           PhaseScope ps(st, PH_SOLUPD, 32.0 * Bn, 2.0 * Bn);
-          HZ_TRY(launch_scale_copy(Vj, sig_j, zt, n, nrhs, ks.active, st));
+          HZ_TRY(launch_scale_copy(W, sig_j, zt, n, nrhs, ks.active, st));
         }
         PhaseScope ps(st, PH_STENCIL, stb, stf);
-        HZ_TRY(launch_stencil(med, 0, zt, n, Vn, n, nrhs, ks.active, st));
+        HZ_TRY(launch_stencil(med, 0, zt, n, W, n, nrhs, ks.active, st));
       } else if (left) {
         // left: v_{j+1} = Q_M (P_N (sigma_j V_j)); the FP64 stencil writes
-        // P_N V_j, the preconditioner scales it by sigma_j and works in place
+        // P_N V_j, which the preconditioner scales by sigma_j
+        double2* zt = static_cast<double2*>(p->Z);
         {
           PhaseScope ps(st, PH_STENCIL, Bn * (16.0 + 32.0 + (med->a ? 8.0 : 0.0)), stf);
-          HZ_TRY(launch_stencil(med, 0, Vj, n, Vn, n, nrhs, ks.active, st));
+          HZ_TRY(launch_stencil(med, 0, W, n, zt, n, nrhs, ks.active, st));
         }
-        HZ_TRY(precond_apply(p, prec, Vn, sig_j, nrhs, Vn, 1, st, ks.active));
+        HZ_TRY(precond_apply(p, prec, zt, sig_j, nrhs, W, 1, st, ks.active));
       } else if (prec == 1) {
         float2* Zj = static_cast<float2*>(p->Z) + long(j) * ldb * n;
-        HZ_TRY(precond_apply(p, 1, Vj, sig_j, nrhs, Zj, 0, st, ks.active));
+        HZ_TRY(precond_apply(p, 1, W, sig_j, nrhs, Zj, 0, st, ks.active));
         PhaseScope ps(st, PH_STENCIL, stb, stf);
-        HZ_TRY(launch_stencil(med, 1, Zj, n, Vn, n, nrhs, ks.active, st));
+        HZ_TRY(launch_stencil(med, 1, Zj, n, W, n, nrhs, ks.active, st));
       } else {
         double2* zt = static_cast<double2*>(p->Z);
-        HZ_TRY(precond_apply(p, 0, Vj, sig_j, nrhs, zt, 1, st, ks.active));
+        HZ_TRY(precond_apply(p, 0, W, sig_j, nrhs, zt, 1, st, ks.active));
         PhaseScope ps(st, PH_STENCIL, stb, stf);
-        HZ_TRY(launch_stencil(med, 0, zt, n, Vn, n, nrhs, ks.active, st));
+        HZ_TRY(launch_stencil(med, 0, zt, n, W, n, nrhs, ks.active, st));
       }
-      // CGS2: two passes of classical Gram-Schmidt against v_0 .. v_j
-      const double db = 16.0 * Bn * (j + 2), ub = 16.0 * Bn * (j + 3), fl = 8.0 * Bn * (j + 1);
-      for (int pass = 0; pass < 2; ++pass) {
-        double2* S = pass == 0 ? ks.S1 : ks.S2;
-        {
-          PhaseScope ps(st, PH_DOTS, db, fl, 2);
-          HZ_TRY(launch_dots(p->V, ldb, Vn, n, n, j, nrhs, ks.active,
-                             reinterpret_cast<double2*>(p->partial), p->tune, S, m + 1, st));
-        }
-        PhaseScope ps(st, PH_UPDATE, ub, fl + (pass ? 4.0 * Bn : 0.0), pass ? 2 : 1);
-        HZ_TRY(launch_update(p->V, ldb, Vn, n, n, j, nrhs, S, m + 1, ks.sigma, B, ks.active, pass == 1,
-                             p->partial, p->tune, ks.nrm2, st));
+      // CGS2: two passes of classical Gram-Schmidt against v_0 .. v_j; the
+      // first update and the second dots are one kernel (counted as dots)
+      const double db = 16.0 * Bn * (j + 2), ub = 16.0 * Bn * (j + 4), fl = 8.0 * Bn * (j + 1);
+      double2* part = reinterpret_cast<double2*>(p->partial);
+      {
+        PhaseScope ps(st, PH_DOTS, db, fl, 2);
+        HZ_TRY(launch_dots(Q, W, n, j, nrhs, ks.active, part, ks.S1, m + 1, st));
+      }
+      {
+        PhaseScope ps(st, PH_DOTS, db + 16.0 * Bn, 2.0 * fl, 2);
+        HZ_TRY(launch_update_dots(Q, W, n, j, nrhs, ks.S1, m + 1, ks.sigma, B, ks.active, part,
+                                  ks.S2, st));
+      }
+      {
+        PhaseScope ps(st, PH_UPDATE, ub, fl + 4.0 * Bn, 2);
+        HZ_TRY(launch_update(Q, W, n, j, nrhs, ks.S2, m + 1, ks.sigma, B, ks.active, p->partial,
+                             ks.nrm2, j + 1 < m, st));
       }
       PhaseScope ps(st, PH_GIVENS, 0.0, 0.0);
       HZ_TRY(launch_givens(ks, j, nrhs, st));
@@ -449,19 +459,17 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
       HZ_TRY(launch_solution_update(1, p->Z, ldb, u, n, n, nrhs, w.y, m, d_jn, st));
     } else if (noq || left) {
       // u += V (sigma y)
-      double2* t = p->V + long(m) * ldb * n;
       PhaseScope ps(st, PH_SOLUPD, Bn * (16.0 * Jmax + 64.0), Bn * (8.0 * Jmax + 2.0));
-      HZ_TRY(launch_combine(p->V, ldb, t, n, n, nrhs, w.y, m, ks.sigma, B, d_jn, st));
-      HZ_TRY(launch_axpy(u, t, n, n, nrhs, d_jn, st));
+      HZ_TRY(launch_combine(Q, W, n, nrhs, w.y, m, ks.sigma, B, d_jn, st));
+      HZ_TRY(launch_axpy(u, W, n, n, nrhs, d_jn, st));
     } else {
       // t = V (sigma y), then u += Q_M t in complex128
-      double2* t = p->V + long(m) * ldb * n;  // V_m is free once the cycle is over
       {
         PhaseScope ps(st, PH_SOLUPD, Bn * (16.0 * Jmax + 16.0), Bn * 8.0 * Jmax);
-        HZ_TRY(launch_combine(p->V, ldb, t, n, n, nrhs, w.y, m, ks.sigma, B, d_jn, st));
+        HZ_TRY(launch_combine(Q, W, n, nrhs, w.y, m, ks.sigma, B, d_jn, st));
       }
       double2* zt = static_cast<double2*>(p->Z);
-      HZ_TRY(precond_apply(p, 0, t, nullptr, nrhs, zt, 1, st, nullptr));
+      HZ_TRY(precond_apply(p, 0, W, nullptr, nrhs, zt, 1, st, nullptr));
       PhaseScope ps(st, PH_SOLUPD, Bn * 48.0, Bn * 2.0);
       HZ_TRY(launch_axpy(u, zt, n, n, nrhs, d_jn, st));
     }
@@ -474,7 +482,7 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
   if (left) {
     {
       PhaseScope ps(st, PH_RESID, 64.0 * Bn + (med->a ? 8.0 * Bn : 0.0), 30.0 * Bn, 2);
-      HZ_TRY(launch_residual(med, u, f, p->V, n, nrhs, nullptr, p->partial, st));
+      HZ_TRY(launch_residual(med, u, f, W, n, nrhs, nullptr, p->partial, st));
       HZ_TRY(launch_reduce_r(p->partial, nblk_r, nrhs, w.rnorm2, st));
     }
     HZ_CUDA(cudaMemcpyAsync(rn2.data(), w.rnorm2, nrhs * sizeof(double), cudaMemcpyDeviceToHost, st));

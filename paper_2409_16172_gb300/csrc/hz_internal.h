@@ -12,6 +12,8 @@
 #define HZ_MAX_K 64     // symbol planes (node bit masks are 64-bit)
 #define HZ_MAX_SEG 72   // interpolation segments incl. the two end entries
 #define HZ_MAX_RESTART 128
+#define HZ_FX_TILE 128  // points of a basis vector that share one exponent
+#define HZ_CGS_BLOCKS 608  // Gram-Schmidt blocks per right-hand side at most (4 times that in all)
 
 namespace hz {
 
@@ -249,12 +251,9 @@ namespace hz {
 struct SolveWs;
 
 // Launch shapes the autotuner chooses per plan (defaults are the untuned
-// choice): blocks per SM of the CGS2 dot and update kernels, basis vectors
-// per dot block, and nodes per block of the last-axis symbol pass.
+// choice): nodes per block of the last-axis symbol pass, form of the
+// x-inverse, columns per thread.
 struct Tune {
-  int dots_bps = 2;
-  int dots_vc = 8;
-  int upd_bps = 4;
   int syminv_kpb = 1;
   int rowinv_mode = 0;  // FftOps::row_inv_acc mode (0..3)
   int col_pair = 1;     // complex64 symbol pass: two columns per thread (2: in
@@ -278,7 +277,10 @@ struct hz_plan {
   void* planes = nullptr;  // [max_nrhs][K][n] in the working precision
   int planes_prec = 1;     // precision the planes buffer is sized for (0 = c128)
   // Krylov workspace (FP64)
-  double2* V = nullptr;    // [(m+1)][max_nrhs][n] unnormalised basis vectors
+  double2* V = nullptr;    // [(m+1)][max_nrhs][n]: slots 0 .. m-1 the unnormalised basis
+                           // vectors in block fixed-point form (16 bytes a point), slot m
+                           // the current vector in FP64
+  int* ev = nullptr;       // [m][max_nrhs][tiles] exponents of the basis tiles
   void* Z = nullptr;       // [m][max_nrhs][n] preconditioned vectors (c64 or unused)
   double2* u = nullptr;    // staged solution for host buffers [max_nrhs][n]
   double2* f = nullptr;    // staged right-hand side for host buffers

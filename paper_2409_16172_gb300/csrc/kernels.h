@@ -89,20 +89,37 @@ hz_status launch_residual(const hz_medium* m, const double2* u, const double2* f
                           cudaStream_t st);
 
 int krylov_blocks(long n, int nrhs, int nchunk);
-hz_status launch_dots(const double2* V, long ldb, const double2* w, long wstride, long n, int j,
-                      int nrhs, const int* active, double2* partial, const Tune& tn, double2* S,
-                      int ldS, cudaStream_t st);
-hz_status launch_update(const double2* V, long ldb, double2* w, long wstride, long n, int j,
-                        int nrhs, const double2* S, int ldS, const double* sigma, int ldsig,
-                        const int* active, bool norm, double* partial, const Tune& tn, double* nrm2,
-                        cudaStream_t st);
+// Arnoldi basis in block fixed-point form (fixed.cuh): vector i of
+// right-hand side b at V + (i ldb + b) n, its tile exponents at
+// ev + (i ldb + b) ntiles.
+struct Basis {
+  int4* V;
+  int* ev;
+  long ldb, n, ntiles;
+};
+// S = raw sums of conj(V_i) w, i <= j (pass 1)
+hz_status launch_dots(const Basis& Q, double2* w, long wstride, int j, int nrhs, const int* active,
+                      double2* partial, double2* S, int ldS, cudaStream_t st);
+// w -= sum_i sigma_i^2 S1_i V_i, then S2 = raw sums of the new w (pass 2)
+hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, int nrhs,
+                             const double2* S1, int ldS, const double* sigma, int ldsig,
+                             const int* active, double2* partial, double2* S2,
+                             cudaStream_t st);
+// w -= sum_i sigma_i^2 S_i V_i and |w|^2; keep: w also becomes V_{j+1}
+hz_status launch_update(const Basis& Q, double2* w, long wstride, int j, int nrhs,
+                        const double2* S, int ldS, const double* sigma, int ldsig,
+                        const int* active, double* partial, double* nrm2,
+                        bool keep, cudaStream_t st);
+// V_i = w
+hz_status launch_encode(const Basis& Q, const double2* w, long wstride, int i, int nrhs,
+                        const int* active, cudaStream_t st);
 hz_status launch_givens(const KsDev& ks, int j, int nrhs, cudaStream_t st);
 hz_status launch_solution_update(int zprec, const void* Z, long ldb, double2* u, long ustride,
                                  long n, int nrhs, const double2* y, int ldy, const int* jn,
                                  cudaStream_t st);
-hz_status launch_combine(const double2* V, long ldb, double2* out, long ostride, long n, int nrhs,
-                         const double2* y, int ldy, const double* sigma, int ldsig, const int* jn,
-                         cudaStream_t st);
+// out = sum_{i < jn[b]} sigma_i y_i V_i
+hz_status launch_combine(const Basis& Q, double2* out, long ostride, int nrhs, const double2* y,
+                         int ldy, const double* sigma, int ldsig, const int* jn, cudaStream_t st);
 hz_status launch_scale_copy(const double2* V, const double* sigma, double2* out, long n, int nrhs,
                            const int* active, cudaStream_t st);
 hz_status launch_axpy(double2* u, const double2* t, long stride, long n, int nrhs, const int* jn,

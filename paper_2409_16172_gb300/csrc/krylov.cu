@@ -8,9 +8,14 @@
 //   h_i   = <v_i, w> = sigma_i * sum conj(V_i) w          (dots)
 //   w    -= sum_i h_i v_i = sum_i (sigma_i h_i) V_i         (update)
 // so no pass ever rescales a stored vector.
-// Layout: V[(i * ldb + b) * n + p] for basis vector i, right-hand side b.
+// Layout: V[(i * ldb + b) * n + p] for basis vector i, right-hand side b, in
+// the block fixed-point form of fixed.cuh (16 bytes a point); the current
+// vector w is FP64.
 #include <math.h>
 
+#include <algorithm>
+
+#include "fixed.cuh"
 #include "hz_internal.h"
 #include "kernels.h"
 
@@ -18,10 +23,9 @@ namespace hz {
 namespace {
 
 constexpr int KT = 256;   // threads per block
-constexpr int VCMAX = 8;  // basis vectors per dots block (at most)
 
 // fixed-order block sum of NV doubles per thread; result in sh[0..NV-1]
-template <int NV>
+template <int NV, int NT = KT>
 __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
 #pragma unroll
   for (int c = 0; c < NV; ++c) {
@@ -36,114 +40,401 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
   __syncthreads();
   if (threadIdx.x < NV) {
     double s = 0.0;
-    for (int w = 0; w < KT / 32; ++w) s += sh[w * NV + threadIdx.x];
-    sh[KT / 32 * NV + threadIdx.x] = s;
+    for (int w = 0; w < NT / 32; ++w) s += sh[w * NV + threadIdx.x];
+    sh[NT / 32 * NV + threadIdx.x] = s;
   }
   __syncthreads();
 }
 
-// S[b][i] partials: raw sums sum_p conj(V_i[p]) w[p] for i in [i0, i0 + nv),
-// chunks of vpc = ceil((j+1) / nchunk) <= VC vectors, i0 = chunk * vpc,
-// nv = min(vpc, j + 1 - i0).  grid = (nblk, nrhs, nchunk).  partial layout
-// [(b * (j+1) + i) * nblk + blk] as double2.  The next point's operands are
-// loaded before the current point's FMAs so that the FP64 pipe, the limit
-// here, does not wait on memory.  With VC <= 4 every product has its own
-// accumulator (re*re, im*im, re*im, im*re), so that no FMA waits on another
-// FMA of the same point; with VC = 8 (register budget) two per vector.  Only
-// the nv live sums are reduced.
-template <int VC> struct DotsCfg {
-  static constexpr int NA = VC <= 4 ? 4 : 2;  // accumulators per vector
-  static constexpr int MINB = VC <= 2 ? 4 : (VC <= 4 ? 3 : 2);
+// ---------------------------------------------------------------------------
+// Gram-Schmidt kernels over the basis in block fixed-point form (fixed.cuh).
+//
+// What bounds them: past about 16 vectors the basis in HBM, 16 bytes a point
+// and vector, before that the work per tile (w to and from integers, folding
+// the sums).  2^24 points: dots 5.4 TB/s of basis at j = 20 and 5.9 at
+// j = 39, update 5.1 and 5.4; in FP64 the same sums were bound by the FP64
+// pipe at 2.1-2.5 TB/s.  A 256^3 Arnoldi step spends 3.7 ms here instead of
+// 9.2.  A
+// block takes one tile of FX_TILE points at a time.  Its basis rows (one row:
+// the tile's 128 points of one vector, 2 KB) come through shared memory by
+// cp.async, so that the loads in flight do not cost registers and run ahead
+// over tile boundaries.
+//   update side  a thread owns a point and runs over the vectors
+//   dot side     the vectors are dealt to the half warps; a lane takes CG_U
+//                points, and the integer sums of CG_NB vectors are folded
+//                across the lanes together before they become doubles
+// ---------------------------------------------------------------------------
+enum CgMode {
+  CG_DOTS = 0,     // partial sums of conj(V_i) w, i <= j
+  CG_UPDATE_DOTS,  // w -= sum_i sigma_i^2 S[b][i] V_i, then the sums of the new w
+  CG_UPDATE,       // w -= ..., |w|^2 sums, the new w as basis vector (unless Vnew is null)
+  CG_COMBINE       // w = sum_i sigma_i S[b][i] V_i, i < jn[b]
 };
 
-template <int VC>
-__global__ void __launch_bounds__(KT, DotsCfg<VC>::MINB)
-dots_kernel(const double2* __restrict__ V, long ldb, const double2* __restrict__ w, long wstride,
-            long n, int j, int vpc, const int* __restrict__ active, double2* __restrict__ partial) {
+constexpr int CT = FX_TILE;               // threads
+constexpr int CG_WARPS = CT / 32;
+constexpr int CG_HALVES = 2 * CG_WARPS;   // vectors in work at a time on the dot side
+constexpr int CG_U = FX_TILE / 16;        // points per lane on the dot side
+constexpr int CG_NB = 4;
+constexpr int CG_ROWS = 24;               // ring rows when rows only pass through
+constexpr int CG_DEPTH = CG_ROWS / CG_HALVES;  // dot side: rows in flight per half warp
+constexpr int CG_NU = 4;                       // update side: rows per copy group
+constexpr int CG_GROUPS = CG_ROWS / CG_NU;     // and groups in flight
+constexpr int CG_MAXROWS = 34;            // ring rows at most (three blocks per SM)
+constexpr int CG_FUSED = 22;              // vectors at most in CG_UPDATE_DOTS
+constexpr size_t CG_ROW_BYTES = FX_TILE * sizeof(int4);
+
+__device__ __forceinline__ void copy16(int4* dst, const int4* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   unsigned(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// sum over the 16 lanes of a half warp of 4 values per lane; lane l returns
+// the sum of value (l >> 2) & 3 (each step sends the half the partner keeps)
+__device__ __forceinline__ long long fold4(const long long (&t)[CG_NB], int lane) {
+  const bool u8 = lane & 8, u4 = lane & 4;
+  long long a = u8 ? t[2] : t[0], b = u8 ? t[3] : t[1];
+  a += __shfl_xor_sync(0xffffffffu, u8 ? t[0] : t[2], 8);
+  b += __shfl_xor_sync(0xffffffffu, u8 ? t[1] : t[3], 8);
+  long long c = u4 ? b : a;
+  c += __shfl_xor_sync(0xffffffffu, u4 ? a : b, 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  return c;
+}
+
+// per-warp maxima into red; the block's maximum after a barrier
+__device__ __forceinline__ void warp_max(int v, int* red) {
+  const int m = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+}
+__device__ __forceinline__ int max_of(const int* red) {
+  int r = red[0];
+#pragma unroll
+  for (int i = 1; i < CG_WARPS; ++i) r = max(r, red[i]);
+  return r;
+}
+
+// exact limb sums of conj(v) y (re, and the two halves of im)
+struct DotAcc {
+  long long rh = 0, rx = 0, rl = 0, ph = 0, px = 0, pl = 0, qh = 0, qx = 0, ql = 0;
+  __device__ __forceinline__ void add(const int4& v, const int4& y) {
+    rh = mad_w(v.z, y.z, mad_w(v.x, y.x, rh));
+    rx = mad_w(v.z, y.w, mad_w(v.w, y.z, mad_w(v.x, y.y, mad_w(v.y, y.x, rx))));
+    rl = mad_w(v.w, y.w, mad_w(v.y, y.y, rl));
+    ph = mad_w(v.x, y.z, ph);
+    px = mad_w(v.x, y.w, mad_w(v.y, y.z, px));
+    pl = mad_w(v.y, y.w, pl);
+    qh = mad_w(v.z, y.x, qh);
+    qx = mad_w(v.z, y.y, mad_w(v.w, y.x, qx));
+    ql = mad_w(v.w, y.y, ql);
+  }
+  // |hh| <= 2^57 over a lane's CG_U points: the sum over 16 lanes fits
+  __device__ __forceinline__ long long re() const { return fx_sum<1>(rh, rx, rl); }
+  __device__ __forceinline__ long long im() const { return fx_sum<1>(ph - qh, px - qx, pl - ql); }
+};
+// exact limb sums of c v
+struct UpdAcc {
+  long long rh = 0, rx = 0, rl = 0, ih = 0, ix = 0, il = 0;
+  __device__ __forceinline__ void add(const int4& c, const int4& v) {
+    const int nh = -c.z, nl = -c.w;
+    rh = mad_w(nh, v.z, mad_w(c.x, v.x, rh));
+    rx = mad_w(nh, v.w, mad_w(nl, v.z, mad_w(c.x, v.y, mad_w(c.y, v.x, rx))));
+    rl = mad_w(nl, v.w, mad_w(c.y, v.y, rl));
+    ih = mad_w(c.z, v.x, mad_w(c.x, v.z, ih));
+    ix = mad_w(c.z, v.y, mad_w(c.w, v.x, mad_w(c.x, v.w, mad_w(c.y, v.z, ix))));
+    il = mad_w(c.w, v.y, mad_w(c.y, v.w, il));
+  }
+  // |hh| <= 2^60 over HZ_MAX_RESTART + 1 vectors
+  __device__ __forceinline__ long long re() const { return fx_sum<2>(rh, rx, rl); }
+  __device__ __forceinline__ long long im() const { return fx_sum<2>(ih, ix, il); }
+};
+
+template <int MODE>
+__global__ void __launch_bounds__(CT, 4)
+cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, long ntiles,
+           double2* __restrict__ w, long wstride, long n, int j, int rows,
+           const double2* __restrict__ S, int ldS, const double* __restrict__ sigma, int ldsig,
+           const int* __restrict__ active, double2* __restrict__ partial, int4* __restrict__ Vnew,
+           int* __restrict__ enew) {
   pdl_wait();
-  constexpr int NA = DotsCfg<VC>::NA;
   const int b = blockIdx.y;
-  const int i0 = blockIdx.z * vpc;
-  const int nv = min(vpc, j + 1 - i0);
-  double acc[NA * VC];
+  if (MODE == CG_COMBINE) {
+    j = active[b] - 1;  // jn
+  } else if (!active[b]) {
+    return;
+  }
+  constexpr bool UPD = MODE != CG_DOTS, DOT = MODE <= CG_UPDATE_DOTS;
+  extern __shared__ int4 ring[];  // [rows][FX_TILE]
+  __shared__ int4 cl[UPD ? HZ_MAX_RESTART : 1];
+  __shared__ int4 wl[DOT ? FX_TILE : 1];
+  __shared__ double2 sacc[DOT ? HZ_MAX_RESTART : 1];
+  __shared__ int redF[CG_WARPS], redw[CG_WARPS];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int hw = tid >> 4, hl = tid & 15;  // half warp, lane of it
+  double2* wb = w + b * wstride;
+  const int4* Vb = V + long(b) * n;
+  const int* eb = ev + long(b) * ntiles;
+  const long vs = ldb * n, es = ldb * ntiles;  // strides between basis vectors
+  const long dt = gridDim.x;
+  long tile = blockIdx.x;
+
+  // ---- update side: coefficients of a tile, as integers of one common unit
+  double2 ci = make_double2(0.0, 0.0);  // thread i holds the coefficient of vector i
+  if (UPD && tid <= j) {
+    const double s = sigma[long(tid) * ldsig + b];
+    const double2 h = S[long(b) * ldS + tid];
+    const double c = MODE == CG_COMBINE ? s : s * s;
+    ci = make_double2(c * h.x, c * h.y);
+  }
+  const int ec = fx_exp(ci);
+  auto tile_exp = [&](long t) { return UPD && tid <= j && t < ntiles ? eb[tid * es + t] : 0; };
+  const int e0 = tile_exp(tile);
+  int F = 0;
+  if (DOT)
+    for (int i = tid; i <= j; i += CT) sacc[i] = make_double2(0.0, 0.0);
+
+  // ---- copies into the ring
+  long qt = tile;  // next to copy: tile qt, row (group) qr of the thread's
+  int qr = 0, qs = 0, rs = 0;
+  // CG_DOTS: the half warp's rows i = hw, hw + 8, ...; a lane copies the
+  // points that it reads
+  const int nr = (j - 2 * warp) / CG_HALVES + 1;  // of the warp's first half (its second: may be one less)
+  auto copy_row = [&] {
+    if (2 * warp <= j && qt < ntiles) {
+      const int i = hw + CG_HALVES * qr;
+      if (i <= j) {
+        int4* d = ring + (hw * CG_DEPTH + qs) * FX_TILE + hl;
+        const int m = int(min(n - qt * FX_TILE, long(FX_TILE))) - hl;
+        const int4* s = Vb + i * vs + qt * FX_TILE + hl;
+        if (m > 16 * (CG_U - 1)) {
 #pragma unroll
-  for (int c = 0; c < NA * VC; ++c) acc[c] = 0.0;
-  const bool on = active[b] != 0;
-  if (on) {
-    const double2* wb = w + b * wstride;
-    const double2* Vb = V + (long(i0) * ldb + b) * n;
-    const long vs = ldb * n;
-    const long step = long(gridDim.x) * KT;
-    long p = long(blockIdx.x) * KT + threadIdx.x;
-    double2 x, v[VC];
-    if (p < n) {
-      x = wb[p];
+          for (int u = 0; u < CG_U; ++u) copy16(d + 16 * u, s + 16 * u);
+        } else {
 #pragma unroll
-      for (int c = 0; c < VC; ++c)
-        if (c < nv) v[c] = Vb[c * vs + p];
-    }
-    while (p < n) {
-      const long q = p + step;
-      double2 xn, vn[VC];
-      if (q < n) {
-        xn = wb[q];
-#pragma unroll
-        for (int c = 0; c < VC; ++c)
-          if (c < nv) vn[c] = Vb[c * vs + q];
-      }
-#pragma unroll
-      for (int c = 0; c < VC; ++c) {
-        if (c < nv) {
-          if constexpr (NA == 4) {
-            acc[4 * c] = fma(v[c].x, x.x, acc[4 * c]);
-            acc[4 * c + 1] = fma(v[c].y, x.y, acc[4 * c + 1]);
-            acc[4 * c + 2] = fma(v[c].x, x.y, acc[4 * c + 2]);
-            acc[4 * c + 3] = fma(v[c].y, x.x, acc[4 * c + 3]);
-          } else {
-            acc[2 * c] = fma(v[c].x, x.x, fma(v[c].y, x.y, acc[2 * c]));
-            acc[2 * c + 1] = fma(v[c].x, x.y, fma(-v[c].y, x.x, acc[2 * c + 1]));
-          }
+          for (int u = 0; u < CG_U; ++u)
+            if (16 * u < m) copy16(d + 16 * u, s + 16 * u);
         }
       }
-      p = q;
-      x = xn;
+      if (++qr == nr) {
+        qr = 0;
+        qt += dt;
+      }
+    }
+    copy_commit();
+    qs = qs + 1 == CG_DEPTH ? 0 : qs + 1;
+  };
+  // update-only modes: the thread's own point, rows in groups of CG_NU
+  const int ng = (j + CG_NU) / CG_NU;  // groups per tile
+  auto copy_group = [&] {
+    if (qt < ntiles) {
+      const long p = qt * FX_TILE + tid;
+      if (p < n) {
+        int4* d = ring + qs * CG_NU * FX_TILE + tid;
+        const int i0 = qr * CG_NU;
+        const int4* s = Vb + i0 * vs + p;
 #pragma unroll
-      for (int c = 0; c < VC; ++c) v[c] = vn[c];
+        for (int u = 0; u < CG_NU; ++u) {
+          if (i0 + u <= j) copy16(d + u * FX_TILE, s);
+          s += vs;
+        }
+      }
+      if (++qr == ng) {
+        qr = 0;
+        qt += dt;
+      }
+    }
+    copy_commit();
+    qs = qs + 1 == CG_GROUPS ? 0 : qs + 1;
+  };
+  // CG_UPDATE_DOTS: all rows of a tile stay until its dots are done; row i of
+  // the block's k-th tile is at ring row (k (j+1) + i) mod rows
+  auto copy_part = [&](long t, int base, int lo, int hi) {  // rows lo <= i < hi of tile t
+    const long p = t * FX_TILE + tid;
+    if (t < ntiles && p < n) {
+      int r = base + lo;
+      r = r >= rows ? r - rows : r;
+      const int4* s = Vb + lo * vs + p;
+#pragma unroll 4
+      for (int i = lo; i < hi; ++i) {
+        copy16(ring + r * FX_TILE + tid, s);
+        s += vs;
+        r = r + 1 == rows ? 0 : r + 1;
+      }
+    }
+    copy_commit();
+  };
+  int base = 0;
+  const int ahead = MODE == CG_UPDATE_DOTS ? min(j + 1, rows - (j + 1)) : 0;
+  if (MODE == CG_DOTS) {
+    for (int k = 0; k < CG_DEPTH; ++k) copy_row();
+  } else if (MODE == CG_UPDATE_DOTS) {
+    copy_part(tile, base, 0, ahead);
+  } else {
+    for (int k = 0; k < CG_GROUPS; ++k) copy_group();
+  }
+  auto load_w = [&](long t) {
+    const long p = t * FX_TILE + tid;
+    return MODE != CG_COMBINE && t < ntiles && p < n ? wb[p] : make_double2(0.0, 0.0);
+  };
+  double2 xn = load_w(tile);
+  if (UPD) {
+    warp_max(tid <= j ? ec + e0 : 0, redF);
+    __syncthreads();
+    F = max_of(redF);
+    if (tid <= j) cl[tid] = fx_pack(ci, F - e0);
+    __syncthreads();
+  }
+
+  double nrm[1] = {0.0};
+  for (; tile < ntiles; tile += dt) {
+    const long p = tile * FX_TILE + tid;
+    const bool in = p < n;
+    double2 x = xn;
+    xn = load_w(tile + dt);
+    const int e1 = tile_exp(tile + dt);
+    if (UPD) {
+      UpdAcc a;
+      if (MODE == CG_UPDATE_DOTS) {
+        // the rest of this tile's rows, and what fits of the next tile's
+        copy_part(tile, base, ahead, j + 1);
+        int nb = base + j + 1;
+        nb = nb >= rows ? nb - rows : nb;
+        copy_part(tile + dt, nb, 0, ahead);
+        copy_wait<2>();
+        int r = base;
+#pragma unroll 2
+        for (int i = 0; i < ahead; ++i) {
+          a.add(cl[i], ring[r * FX_TILE + tid]);
+          r = r + 1 == rows ? 0 : r + 1;
+        }
+        copy_wait<1>();
+#pragma unroll 2
+        for (int i = ahead; i <= j; ++i) {
+          a.add(cl[i], ring[r * FX_TILE + tid]);
+          r = r + 1 == rows ? 0 : r + 1;
+        }
+      } else {
+        for (int k = 0; k < ng; ++k) {
+          copy_wait<CG_GROUPS - 1>();
+          const int i0 = k * CG_NU;
+          const int4* s = ring + rs * CG_NU * FX_TILE + tid;
+          if (i0 + CG_NU <= j + 1) {
+#pragma unroll
+            for (int u = 0; u < CG_NU; ++u) a.add(cl[i0 + u], s[u * FX_TILE]);
+          } else {
+#pragma unroll
+            for (int u = 0; u < CG_NU; ++u)
+              if (i0 + u <= j) a.add(cl[i0 + u], s[u * FX_TILE]);
+          }
+          copy_group();
+          rs = rs + 1 == CG_GROUPS ? 0 : rs + 1;
+        }
+      }
+      const int k = fx_unit<2>(F);
+      const double dr = fx_to(a.re(), k), di = fx_to(a.im(), k);
+      x = MODE == CG_COMBINE ? make_double2(dr, di) : make_double2(x.x - dr, x.y - di);
+      if (in) wb[p] = x;
+      else x = make_double2(0.0, 0.0);
+      if (MODE == CG_UPDATE) nrm[0] = fma(x.x, x.x, fma(x.y, x.y, nrm[0]));
+      warp_max(tid <= j ? ec + e1 : 0, redF);
+    }
+    if (MODE != CG_COMBINE) warp_max(fx_exp(x), redw);
+    __syncthreads();
+    if (UPD) {
+      F = max_of(redF);
+      if (tid <= j) cl[tid] = fx_pack(ci, F - e1);
+    }
+    const int E = MODE != CG_COMBINE ? max_of(redw) : 0;
+    if (MODE == CG_UPDATE && Vnew) {
+      if (in) Vnew[long(b) * n + p] = fx_pack(x, E);
+      if (tid == 0) enew[long(b) * ntiles + tile] = E;
+    }
+    if (DOT) wl[tid] = fx_pack(x, E);
+    __syncthreads();
+    if (DOT) {
+      int4 wr[CG_U];
+#pragma unroll
+      for (int u = 0; u < CG_U; ++u) wr[u] = wl[u * 16 + hl];
+      for (int i0 = 2 * warp; i0 <= j; i0 += CG_HALVES * CG_NB) {
+        const int is = i0 + (hw & 1) + CG_HALVES * ((lane >> 2) & 3);  // whose sum this lane gets
+        const int e = is <= j ? eb[is * es + tile] : 0;
+        long long tr[CG_NB], ti[CG_NB];
+#pragma unroll
+        for (int c = 0; c < CG_NB; ++c) {
+          tr[c] = ti[c] = 0;
+          if (i0 + CG_HALVES * c <= j) {  // the warp's first half; a second half past j sums what is not used
+            int r;
+            if (MODE == CG_DOTS) {
+              copy_wait<CG_DEPTH - 1>();
+              r = hw * CG_DEPTH + rs;
+            } else {
+              r = base + min(i0 + (hw & 1) + CG_HALVES * c, j);
+              r = r >= rows ? r - rows : r;
+            }
+            const int4* s = ring + r * FX_TILE + hl;
+            DotAcc a;
+            // points past the end: wr is zero there, whatever the ring holds
+#pragma unroll
+            for (int u = 0; u < CG_U; ++u) a.add(s[16 * u], wr[u]);
+            tr[c] = a.re();
+            ti[c] = a.im();
+            if (MODE == CG_DOTS) {
+              copy_row();
+              rs = rs + 1 == CG_DEPTH ? 0 : rs + 1;
+            }
+          }
+        }
+        const long long sr = fold4(tr, lane), si = fold4(ti, lane);
+        if ((lane & 3) == 0 && is <= j) {
+          const int k = fx_unit<1>(E + e);
+          double2 s = sacc[is];
+          s.x += fx_to(sr, k);
+          s.y += fx_to(si, k);
+          sacc[is] = s;
+        }
+      }
+      if (MODE == CG_UPDATE_DOTS) {
+        base += j + 1;
+        base = base >= rows ? base - rows : base;
+        __syncthreads();  // the tile's rows are free
+      }
     }
   }
-  // conj(v) x = (re re + im im) + i (re im - im re)
-  double sum[2 * VC];
-#pragma unroll
-  for (int c = 0; c < VC; ++c) {
-    if constexpr (NA == 4) {
-      sum[2 * c] = acc[4 * c] + acc[4 * c + 1];
-      sum[2 * c + 1] = acc[4 * c + 2] - acc[4 * c + 3];
-    } else {
-      sum[2 * c] = acc[2 * c];
-      sum[2 * c + 1] = acc[2 * c + 1];
-    }
+  copy_wait<0>();
+  if (DOT) {
+    __syncthreads();
+    for (int i = tid; i <= j; i += CT)
+      partial[(long(b) * (j + 1) + i) * gridDim.x + blockIdx.x] = sacc[i];
   }
-  // block reduction of the 2 nv live sums (warp shuffles, then one value per warp)
-  __shared__ double sh[(KT / 32) * 2 * VC];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int c = 0; c < 2 * VC; ++c) {
-    if (c < 2 * nv) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum[c] += __shfl_down_sync(0xffffffffu, sum[c], o);
-      if (lane == 0) sh[warp * 2 * VC + c] = sum[c];
-    }
+  if (MODE == CG_UPDATE) {
+    __shared__ double sh[KT / 32 + 1];
+    block_sum<1, CT>(nrm, sh);
+    if (tid == 0)
+      reinterpret_cast<double*>(partial)[long(b) * gridDim.x + blockIdx.x] = sh[CT / 32];
   }
+}
+
+// w as basis vector: the first one of a cycle
+__global__ void __launch_bounds__(CT)
+encode_kernel(const double2* __restrict__ w, long wstride, long n, long ntiles,
+              const int* __restrict__ active, int4* __restrict__ V, int* __restrict__ ev) {
+  pdl_wait();
+  const int b = blockIdx.y;
+  if (!active[b]) return;
+  __shared__ int red[CG_WARPS];
+  const long p = long(blockIdx.x) * FX_TILE + threadIdx.x;
+  const double2 x = p < n ? w[b * wstride + p] : make_double2(0.0, 0.0);
+  warp_max(fx_exp(x), red);
   __syncthreads();
-  if (threadIdx.x < 2 * nv) {
-    double s = 0.0;
-    for (int wi = 0; wi < KT / 32; ++wi) s += sh[wi * 2 * VC + threadIdx.x];
-    sh[threadIdx.x] = s;  // rows 0..: warp 0's slots are no longer needed
-  }
-  __syncthreads();
-  if (threadIdx.x < nv)
-    partial[(long(b) * (j + 1) + i0 + threadIdx.x) * gridDim.x + blockIdx.x] =
-        make_double2(sh[2 * threadIdx.x], sh[2 * threadIdx.x + 1]);
+  const int E = max_of(red);
+  if (p < n) V[long(b) * n + p] = fx_pack(x, E);
+  if (threadIdx.x == 0) ev[long(b) * ntiles + blockIdx.x] = E;
 }
 
 // Sum partials in a fixed order: q = b * jp1 + i,
@@ -174,66 +465,6 @@ reduce_r_kernel(const double* __restrict__ part, int nblk, double* __restrict__ 
   __shared__ double sh[(KT / 32 + 1)];
   block_sum<1>(v, sh);
   if (threadIdx.x == 0) out[q] = sh[KT / 32];
-}
-
-// w -= sum_{i <= j} sigma_i^2 S[b][i] V_i, optionally |w|^2 partials.
-template <bool NORM>
-__global__ void __launch_bounds__(KT)
-update_kernel(const double2* __restrict__ V, long ldb, double2* __restrict__ w, long wstride,
-              long n, int j, const double2* __restrict__ S, int ldS, const double* __restrict__ sigma,
-              int ldsig, const int* __restrict__ active, double* __restrict__ partial) {
-  pdl_wait();
-  const int b = blockIdx.y;
-  __shared__ double2 coef[HZ_MAX_RESTART + 1];
-  const bool on = active[b] != 0;
-  if (on) {
-    for (int i = threadIdx.x; i <= j; i += KT) {
-      const double s = sigma[long(i) * ldsig + b];
-      const double2 h = S[long(b) * ldS + i];
-      coef[i] = make_double2(s * s * h.x, s * s * h.y);
-    }
-  }
-  __syncthreads();
-  double nrm[1] = {0.0};
-  if (on) {
-    double2* wb = w + b * wstride;
-    const double2* Vb = V + long(b) * n;
-    const long vs = ldb * n;  // stride between basis vectors
-    for (long p = long(blockIdx.x) * KT + threadIdx.x; p < n; p += long(gridDim.x) * KT) {
-      // d = sum_i c_i V_i[p] in two interleaved partial sums; loads hoisted
-      double dr0 = 0.0, di0 = 0.0, dr1 = 0.0, di1 = 0.0;
-      int i = 0;
-      for (; i + 3 <= j; i += 4) {
-        const double2 v0 = Vb[(i + 0) * vs + p], v1 = Vb[(i + 1) * vs + p];
-        const double2 v2 = Vb[(i + 2) * vs + p], v3 = Vb[(i + 3) * vs + p];
-        const double2 c0 = coef[i], c1 = coef[i + 1], c2 = coef[i + 2], c3 = coef[i + 3];
-        dr0 = fma(c0.x, v0.x, fma(-c0.y, v0.y, dr0));
-        di0 = fma(c0.x, v0.y, fma(c0.y, v0.x, di0));
-        dr1 = fma(c1.x, v1.x, fma(-c1.y, v1.y, dr1));
-        di1 = fma(c1.x, v1.y, fma(c1.y, v1.x, di1));
-        dr0 = fma(c2.x, v2.x, fma(-c2.y, v2.y, dr0));
-        di0 = fma(c2.x, v2.y, fma(c2.y, v2.x, di0));
-        dr1 = fma(c3.x, v3.x, fma(-c3.y, v3.y, dr1));
-        di1 = fma(c3.x, v3.y, fma(c3.y, v3.x, di1));
-      }
-      for (; i <= j; ++i) {
-        const double2 v = Vb[i * vs + p];
-        const double2 c = coef[i];
-        dr0 = fma(c.x, v.x, fma(-c.y, v.y, dr0));
-        di0 = fma(c.x, v.y, fma(c.y, v.x, di0));
-      }
-      double2 x = wb[p];
-      x.x -= dr0 + dr1;
-      x.y -= di0 + di1;
-      wb[p] = x;
-      if (NORM) nrm[0] = fma(x.x, x.x, fma(x.y, x.y, nrm[0]));
-    }
-  }
-  if (NORM) {
-    __shared__ double sh[KT / 32 + 1];
-    block_sum<1>(nrm, sh);
-    if (threadIdx.x == 0) partial[long(b) * gridDim.x + blockIdx.x] = sh[KT / 32];
-  }
 }
 
 __device__ __forceinline__ double2 cmul_d(double2 a, double2 b) {
@@ -438,35 +669,6 @@ solution_update_kernel(const ZT* __restrict__ Z, long ldb, double2* __restrict__
   }
 }
 
-// out[b] = sum_{i < J} (sigma_i y_i) V_i  (FP64 path: the combination that is
-// then preconditioned).
-__global__ void __launch_bounds__(KT)
-combine_kernel(const double2* __restrict__ V, long ldb, double2* __restrict__ out, long ostride,
-               long n, const double2* __restrict__ y, int ldy, const double* __restrict__ sigma,
-               int ldsig, const int* __restrict__ jn) {
-  pdl_wait();
-  const int b = blockIdx.y;
-  const int J = jn[b];
-  __shared__ double2 ys[HZ_MAX_RESTART];
-  for (int i = threadIdx.x; i < J; i += KT) {
-    const double s = sigma[long(i) * ldsig + b];
-    const double2 yy = y[long(b) * ldy + i];
-    ys[i] = make_double2(s * yy.x, s * yy.y);
-  }
-  __syncthreads();
-  double2* ob = out + b * ostride;
-  for (long p = long(blockIdx.x) * KT + threadIdx.x; p < n; p += long(gridDim.x) * KT) {
-    double2 x = make_double2(0.0, 0.0);
-    for (int i = 0; i < J; ++i) {
-      const double2 v = V[(long(i) * ldb + b) * n + p];
-      const double2 c = ys[i];
-      x.x = fma(c.x, v.x, fma(-c.y, v.y, x.x));
-      x.y = fma(c.x, v.y, fma(c.y, v.x, x.y));
-    }
-    ob[p] = x;
-  }
-}
-
 // u += t (element-wise, FP64), for active right-hand sides with jn > 0
 __global__ void axpy_kernel(double2* __restrict__ u, const double2* __restrict__ t, long stride,
                             long n, const int* __restrict__ jn) {
@@ -524,48 +726,93 @@ int krylov_blocks_bps(long n, int nrhs, int nchunk, int bps) {
 
 int krylov_blocks(long n, int nrhs, int nchunk) { return krylov_blocks_bps(n, nrhs, nchunk, 4); }
 
-hz_status launch_dots(const double2* V, long ldb, const double2* w, long wstride, long n, int j,
-                      int nrhs, const int* active, double2* partial, const Tune& tn, double2* S,
-                      int ldS, cudaStream_t st) {
-  // balanced chunks of at most vc vectors; one wave of tn.dots_bps blocks
-  // per SM (the register budget allows two)
-  const int vc = tn.dots_vc <= 2 ? 2 : (tn.dots_vc <= 4 ? 4 : VCMAX);
-  int nchunk = (j + 1 + vc - 1) / vc;
-  const int vpc = (j + 1 + nchunk - 1) / nchunk;
-  nchunk = (j + 1 + vpc - 1) / vpc;  // no empty chunk
-  long per = (long(tn.dots_bps) * 152) / (long(nrhs) * nchunk);
-  const long cap = (n + KT - 1) / KT;  // at least one point per thread
-  if (per > cap) per = cap;
-  const int nblk = int(per < 1 ? 1 : per);
-  if (vc == 2)
-    HZ_CUDA(launch_pdl(dots_kernel<2>, dim3(nblk, nrhs, nchunk), dim3(KT), 0, st, V, ldb, w,
-                       wstride, n, j, vpc, active, partial));
-  else if (vc == 4)
-    HZ_CUDA(launch_pdl(dots_kernel<4>, dim3(nblk, nrhs, nchunk), dim3(KT), 0, st, V, ldb, w,
-                       wstride, n, j, vpc, active, partial));
-  else
-    HZ_CUDA(launch_pdl(dots_kernel<VCMAX>, dim3(nblk, nrhs, nchunk), dim3(KT), 0, st, V, ldb, w,
-                       wstride, n, j, vpc, active, partial));
+namespace {
+// Blocks per right-hand side of the Gram-Schmidt kernels: they walk over the
+// tiles, so per_sm * 152 blocks are asked for (what fits at a time); with
+// several right-hand sides as many whole waves as leave the fewest SMs idle.
+int cgs_blocks(long ntiles, int nrhs, int per_sm) {
+  const long wave = long(per_sm) * 152;
+  long best = 1;
+  double fill = 0.0;
+  for (int k = 1; k <= 4; ++k) {
+    const long per = k * wave / nrhs;
+    const double f = double(per) * nrhs / double(k * wave);
+    if (per >= 1 && f > fill + 0.03) {
+      fill = f;
+      best = per;
+    }
+  }
+  return int(std::min(std::min(best, long(HZ_CGS_BLOCKS)), ntiles));
+}
+
+template <int MODE>
+hz_status launch_cgs(const Basis& Q, int nblk, int rows, double2* w, long wstride, int j, int nrhs,
+                     const double2* S, int ldS, const double* sigma, int ldsig, const int* active,
+                     double2* partial, int4* Vnew, int* enew, cudaStream_t st) {
+  // one limit for every launch: other threads may be launching the same kernel
+  // with another number of rows
+  constexpr int limit = int((MODE == CG_UPDATE_DOTS ? CG_MAXROWS : CG_ROWS) * CG_ROW_BYTES);
+  HZ_CUDA(cudaFuncSetAttribute(cgs_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+  HZ_CUDA(launch_pdl(cgs_kernel<MODE>, dim3(nblk, nrhs), dim3(CT), rows * CG_ROW_BYTES, st, Q.V,
+                     Q.ev, Q.ldb, Q.ntiles, w, wstride, Q.n, j, rows, S, ldS, sigma, ldsig, active, partial,
+                     Vnew, enew));
+  return HZ_OK;
+}
+}  // namespace
+
+hz_status launch_dots(const Basis& Q, double2* w, long wstride, int j, int nrhs, const int* active,
+                      double2* partial, double2* S, int ldS, cudaStream_t st) {
+  const int nblk = cgs_blocks(Q.ntiles, nrhs, 4);
+  HZ_TRY(launch_cgs<CG_DOTS>(Q, nblk, CG_ROWS, w, wstride, j, nrhs, nullptr, 0, nullptr, 0, active, partial,
+                             nullptr, nullptr, st));
   HZ_CUDA(launch_pdl(reduce_c_kernel, dim3(unsigned(nrhs * (j + 1))), dim3(KT), 0, st, partial,
                      nblk, j + 1, ldS, S));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
 }
 
-hz_status launch_update(const double2* V, long ldb, double2* w, long wstride, long n, int j,
-                        int nrhs, const double2* S, int ldS, const double* sigma, int ldsig,
-                        const int* active, bool norm, double* partial, const Tune& tn, double* nrm2,
-                        cudaStream_t st) {
-  const int nblk = krylov_blocks_bps(n, nrhs, 1, tn.upd_bps);
-  if (norm) {
-    HZ_CUDA(launch_pdl(update_kernel<true>, dim3(nblk, nrhs), dim3(KT), 0, st, V, ldb, w, wstride,
-                       n, j, S, ldS, sigma, ldsig, active, partial));
-    HZ_CUDA(launch_pdl(reduce_r_kernel, dim3(unsigned(nrhs)), dim3(KT), 0, st, partial, nblk,
-                       nrm2));
-  } else {
-    HZ_CUDA(launch_pdl(update_kernel<false>, dim3(nblk, nrhs), dim3(KT), 0, st, V, ldb, w, wstride,
-                       n, j, S, ldS, sigma, ldsig, active, nullptr));
+hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, int nrhs,
+                             const double2* S1, int ldS, const double* sigma, int ldsig,
+                             const int* active, double2* partial, double2* S2,
+                             cudaStream_t st) {
+  // One kernel while a tile's rows and part of the next tile's fit the shared
+  // memory of a third of an SM; past that its few warps cost more than the
+  // second read of the basis (2^24 points: j = 9 1112 us against 1238 us in
+  // two kernels, j = 20 2104 against 2153, j = 39 4203 against 3806).
+  if (j + 1 > CG_FUSED) {
+    HZ_TRY(launch_cgs<CG_UPDATE>(Q, cgs_blocks(Q.ntiles, nrhs, 4), CG_ROWS, w, wstride, j, nrhs,
+                                 S1, ldS, sigma, ldsig, active, partial, nullptr, nullptr, st));
+    return launch_dots(Q, w, wstride, j, nrhs, active, partial, S2, ldS, st);
   }
+  const int per_sm = j + 1 <= 16 ? 4 : 3;
+  const int rows = per_sm == 4 ? CG_ROWS : CG_MAXROWS;
+  const int nblk = cgs_blocks(Q.ntiles, nrhs, per_sm);
+  HZ_TRY(launch_cgs<CG_UPDATE_DOTS>(Q, nblk, rows, w, wstride, j, nrhs, S1, ldS, sigma, ldsig,
+                                    active, partial, nullptr, nullptr, st));
+  HZ_CUDA(launch_pdl(reduce_c_kernel, dim3(unsigned(nrhs * (j + 1))), dim3(KT), 0, st, partial,
+                     nblk, j + 1, ldS, S2));
+  HZ_CUDA(cudaGetLastError());
+  return HZ_OK;
+}
+
+hz_status launch_update(const Basis& Q, double2* w, long wstride, int j, int nrhs,
+                        const double2* S, int ldS, const double* sigma, int ldsig,
+                        const int* active, double* partial, double* nrm2,
+                        bool keep, cudaStream_t st) {
+  const int nblk = cgs_blocks(Q.ntiles, nrhs, 4);
+  HZ_TRY(launch_cgs<CG_UPDATE>(Q, nblk, CG_ROWS, w, wstride, j, nrhs, S, ldS, sigma, ldsig, active,
+                               reinterpret_cast<double2*>(partial),
+                               keep ? Q.V + (j + 1) * Q.ldb * Q.n : nullptr,
+                               keep ? Q.ev + (j + 1) * Q.ldb * Q.ntiles : nullptr, st));
+  HZ_CUDA(launch_pdl(reduce_r_kernel, dim3(unsigned(nrhs)), dim3(KT), 0, st, partial, nblk, nrm2));
+  HZ_CUDA(cudaGetLastError());
+  return HZ_OK;
+}
+
+hz_status launch_encode(const Basis& Q, const double2* w, long wstride, int i, int nrhs,
+                        const int* active, cudaStream_t st) {
+  HZ_CUDA(launch_pdl(encode_kernel, dim3(unsigned(Q.ntiles), nrhs), dim3(CT), 0, st, w, wstride,
+                     Q.n, Q.ntiles, active, Q.V + i * Q.ldb * Q.n, Q.ev + i * Q.ldb * Q.ntiles));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
 }
@@ -590,12 +837,10 @@ hz_status launch_solution_update(int zprec, const void* Z, long ldb, double2* u,
   return HZ_OK;
 }
 
-hz_status launch_combine(const double2* V, long ldb, double2* out, long ostride, long n, int nrhs,
-                         const double2* y, int ldy, const double* sigma, int ldsig, const int* jn,
-                         cudaStream_t st) {
-  const int nblk = krylov_blocks(n, nrhs, 1);
-  HZ_CUDA(launch_pdl(combine_kernel, dim3(nblk, nrhs), dim3(KT), 0, st, V, ldb, out, ostride, n, y,
-                     ldy, sigma, ldsig, jn));
+hz_status launch_combine(const Basis& Q, double2* out, long ostride, int nrhs, const double2* y,
+                         int ldy, const double* sigma, int ldsig, const int* jn, cudaStream_t st) {
+  HZ_TRY(launch_cgs<CG_COMBINE>(Q, cgs_blocks(Q.ntiles, nrhs, 4), CG_ROWS, out, ostride, 0, nrhs, y, ldy,
+                                sigma, ldsig, jn, nullptr, nullptr, nullptr, st));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
 }

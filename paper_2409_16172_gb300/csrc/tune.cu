@@ -2,13 +2,11 @@
 // solve by timing the candidates on the plan's own buffers, once per
 // (grid, K, right-hand sides, restart, precision) in a process, and caches
 // the choice.  Candidates:
-//   CGS2 dot kernel   (vectors per block, blocks per SM) in
-//                     {(8, 1), (8, 2), (4, 2), (4, 3), (2, 2), (2, 4)}
-//   CGS2 update       blocks per SM {2, 4, 6, 8}
 //   symbol pass       nodes per block {1, 2, 4} (the spectrum is read once
 //                     per block; fewer, longer blocks), one or two columns
 //                     per thread (complex64)
 //   x-inverse pass    fused weighted sum, or in place + gather
+// The Gram-Schmidt kernels have one launch shape; their times are reported.
 // Timing uses CUDA events on the caller's stream around 3 repetitions of
 // each candidate at the middle Arnoldi step of a cycle.
 #include <algorithm>
@@ -66,6 +64,13 @@ struct Timer {
   }
 };
 
+// the report's fields of the Gram-Schmidt kernels' fixed shape
+void gs_shape(hz_tune_report* r) {
+  r->dots_bps = 4;
+  r->dots_vc = 8;
+  r->upd_bps = 4;
+}
+
 }  // namespace
 
 // Launch shapes from the process cache without timing: the entry of the
@@ -100,15 +105,11 @@ bool hz::tune_from_cache(hz_plan* plan) {
 
 extern "C" hz_status hz_plan_set_tune(hz_plan* plan, const hz_tune_report* r) {
   if (!plan || !r) return set_error(HZ_ERR_INVALID_ARG, "null argument");
-  // the plan's partial-sum buffer is sized for these ranges
   const bool ok = (r->dots_vc == 2 || r->dots_vc == 4 || r->dots_vc == 8) && r->dots_bps >= 1 &&
                   r->dots_bps <= 4 && r->upd_bps >= 1 && r->upd_bps <= 8 &&
                   (r->syminv_kpb == 1 || r->syminv_kpb == 2 || r->syminv_kpb == 4) &&
                   r->rowinv_mode >= 0 && r->rowinv_mode <= 3 && r->col_pair >= 0 && r->col_pair <= 2;
   if (!ok) return set_error(HZ_ERR_INVALID_ARG, "launch shape out of range");
-  plan->tune.dots_vc = r->dots_vc;
-  plan->tune.dots_bps = r->dots_bps;
-  plan->tune.upd_bps = r->upd_bps;
   plan->tune.syminv_kpb = r->syminv_kpb;
   plan->tune.rowinv_mode = r->rowinv_mode;
   plan->tune.col_pair = r->col_pair;
@@ -125,9 +126,7 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
       plan->tune = it->second;
       if (rep) {
         *rep = hz_tune_report{};
-        rep->dots_bps = plan->tune.dots_bps;
-        rep->dots_vc = plan->tune.dots_vc;
-        rep->upd_bps = plan->tune.upd_bps;
+        gs_shape(rep);
         rep->syminv_kpb = plan->tune.syminv_kpb;
         rep->rowinv_mode = plan->tune.rowinv_mode;
         rep->col_pair = plan->tune.col_pair;
@@ -146,64 +145,35 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
   const long ldb = B;
   KsDev& ks = p->ws->ks;
   // defined contents for the timed kernels: zero basis, unit scales, all active
-  HZ_CUDA(cudaMemsetAsync(p->V, 0, size_t(j + 2) * B * n * sizeof(double2), st));
+  const Basis Q{reinterpret_cast<int4*>(p->V), p->ev, ldb, n, (n + HZ_FX_TILE - 1) / HZ_FX_TILE};
+  double2* W = p->V + long(m) * ldb * n;
+  HZ_CUDA(cudaMemsetAsync(p->V, 0, size_t(j + 1) * B * n * sizeof(double2), st));
+  HZ_CUDA(cudaMemsetAsync(W, 0, size_t(B) * n * sizeof(double2), st));
+  HZ_CUDA(cudaMemsetAsync(p->ev, 0, size_t(j + 1) * B * Q.ntiles * sizeof(int), st));
   HZ_CUDA(cudaMemsetAsync(ks.sigma, 0, size_t(m + 1) * B * sizeof(double), st));
   HZ_CUDA(cudaMemsetAsync(ks.S1, 0, size_t(m + 1) * B * sizeof(double2), st));
   std::vector<int> ones(B, 1);
   HZ_CUDA(cudaMemcpyAsync(ks.active, ones.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
   HZ_CUDA(cudaMemsetAsync(p->tmp, 0, size_t(B) * n * 16, st));
   HZ_CUDA(cudaStreamSynchronize(st));
-  double2* Vn = p->V + long(j + 1) * ldb * n;
   Timer tm(st);
   const Tune def;
   Tune best = def;
   hz_tune_report r{};
 
-  // CGS2 dot products
-  float tbest = 1e30f, tdef = 0.f;
-  const int cand[6][2] = {{8, 1}, {8, 2}, {4, 2}, {4, 3}, {2, 2}, {2, 4}};
-  for (const auto& c : cand) {
-    const int vc = c[0], bps = c[1];
-    {
-      Tune t = best;
-      t.dots_bps = bps;
-      t.dots_vc = vc;
-      const float ms = tm.best_ms([&] {
-        return launch_dots(p->V, ldb, Vn, n, n, j, B, ks.active,
-                           reinterpret_cast<double2*>(p->partial), t, ks.S1, m + 1, st);
-      });
-      if (bps == def.dots_bps && vc == def.dots_vc) tdef = ms;
-      if (ms < tbest) {
-        tbest = ms;
-        best.dots_bps = bps;
-        best.dots_vc = vc;
-      }
-    }
-  }
-  r.dots_us = 1e3f * tbest;
-  r.dots_us_default = 1e3f * tdef;
-
-  // CGS2 update
-  tbest = 1e30f;
-  for (int bps : {2, 4, 6, 8}) {
-    Tune t = best;
-    t.upd_bps = bps;
-    const float ms = tm.best_ms([&] {
-      return launch_update(p->V, ldb, Vn, n, n, j, B, ks.S1, m + 1, ks.sigma, B, ks.active, false,
-                           p->partial, t, ks.nrm2, st);
-    });
-    if (bps == def.upd_bps) tdef = ms;
-    if (ms < tbest) {
-      tbest = ms;
-      best.upd_bps = bps;
-    }
-  }
-  r.upd_us = 1e3f * tbest;
-  r.upd_us_default = 1e3f * tdef;
+  // Gram-Schmidt kernels
+  r.dots_us = r.dots_us_default = 1e3f * tm.best_ms([&] {
+    return launch_dots(Q, W, n, j, B, ks.active, reinterpret_cast<double2*>(p->partial), ks.S1,
+                       m + 1, st);
+  });
+  r.upd_us = r.upd_us_default = 1e3f * tm.best_ms([&] {
+    return launch_update(Q, W, n, j, B, ks.S1, m + 1, ks.sigma, B, ks.active, p->partial, ks.nrm2,
+                         false, st);
+  });
 
   // symbol pass, through a whole preconditioner apply (its other passes do
   // not depend on the choice)
-  tbest = 1e30f;
+  float tbest = 1e30f, tdef = 0.f;
   const int prec = p->opts.precision;
   void* out = p->Z;
   for (int pair : {1, 2, 0}) {
@@ -214,7 +184,7 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
       p->tune.syminv_kpb = kpb;
       p->tune.col_pair = pair;
       const float ms = tm.best_ms([&] {
-        return precond_apply(p, prec, p->V, nullptr, B, out, prec == 1 ? 0 : 1, st, nullptr);
+        return precond_apply(p, prec, W, nullptr, B, out, prec == 1 ? 0 : 1, st, nullptr);
       });
       if (kpb == def.syminv_kpb && pair == def.col_pair) tdef = ms;
       if (ms < tbest) {
@@ -233,7 +203,7 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
     p->tune = best;
     p->tune.rowinv_mode = mode;
     const float ms = tm.best_ms([&] {
-      return precond_apply(p, prec, p->V, nullptr, B, out, prec == 1 ? 0 : 1, st, nullptr);
+      return precond_apply(p, prec, W, nullptr, B, out, prec == 1 ? 0 : 1, st, nullptr);
     });
     if (ms < tbest) {
       tbest = ms;
@@ -244,9 +214,7 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
   r.apply_us_default = 1e3f * tdef;
   HZ_CUDA(cudaStreamSynchronize(st));
   p->tune = best;
-  r.dots_bps = best.dots_bps;
-  r.dots_vc = best.dots_vc;
-  r.upd_bps = best.upd_bps;
+  gs_shape(&r);
   r.syminv_kpb = best.syminv_kpb;
   r.rowinv_mode = best.rowinv_mode;
   r.col_pair = best.col_pair;
