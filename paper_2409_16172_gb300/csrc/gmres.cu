@@ -153,7 +153,7 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
   if (!f_dev) HZ_CUDA(cudaMemcpyAsync(p->f, f_in, vbytes, cudaMemcpyHostToDevice, st));
   if (!u_dev) HZ_CUDA(cudaMemcpyAsync(p->u, u_io, vbytes, cudaMemcpyHostToDevice, st));
 
-  const int nblk_r = stencil_blocks(n);
+  const int nblk_r = stencil_blocks(med);
   const int nblk_n = krylov_blocks(n, nrhs, 1);
   const double Bn = double(nrhs) * n;
   {

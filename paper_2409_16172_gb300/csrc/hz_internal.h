@@ -143,7 +143,10 @@ struct hz_medium {
   std::vector<double> a_nodes;
   // device data
   hz::DevArena arena;
-  double2* gamma2 = nullptr;        // per point gamma^2 / h_x^2 (Eqn. Complex_wave_speed squared)
+  double2* gamma2 = nullptr;        // per point gamma^2 / h_x^2 (Eqn. Complex_wave_speed squared);
+                                    // gfix: as integers of 2^gunit in 31-bit limbs (int4)
+  bool gfix = false;
+  int gunit = 0;
   double* a = nullptr;              // per point operator damping (NULL when a == 0)
   double* rec64 = nullptr;          // per point segment + t (complex128 path)
   uint32_t* rec32 = nullptr;        // per point segment:8 | t:24 (complex64 path)

@@ -80,7 +80,9 @@ struct BatchCtl {
 hz_status gmres_batch(hz_plan* plan, cudaStream_t st,
                       const std::function<int(BatchCtl&)>& boundary);
 
-int stencil_blocks(long n);
+// blocks (partial sums of the residual) per right-hand side
+int stencil_blocks(const hz_medium* m);
+hz_status stencil_prepare(hz_medium* m, double zeta_max, cudaStream_t st);
 hz_status launch_stencil(const hz_medium* m, int in_prec, const void* x, long in_stride,
                          double2* y, long out_stride, int nrhs, const int* active,
                          cudaStream_t st);

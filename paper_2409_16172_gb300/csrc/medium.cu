@@ -10,6 +10,7 @@
 #include <cmath>
 
 #include "hz_internal.h"
+#include "kernels.h"
 
 namespace hz {
 namespace {
@@ -648,6 +649,7 @@ extern "C" hz_status hz_create_medium(const hz_grid* grid, const double* c, cons
     const double h = m->L / N;
     m->inv_h2[d] = 1.0 / (h * h);
   }
+  if ((st = stencil_prepare(m, zmax, cs)) != HZ_OK) return fail(st);
   ce = cudaStreamSynchronize(cs);
   if (ce != cudaSuccess) return fail(cuda_error(ce, "create_medium"));
   *out = m;
