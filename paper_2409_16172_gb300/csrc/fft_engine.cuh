@@ -552,34 +552,6 @@ template <> struct ColPlan<float, 512> { using P = FftPlanW<512>; };
 template <typename R, int N> struct PairPlan { using P = typename ColPlan<R, N>::P; };
 template <> struct PairPlan<float, 1024> { using P = FftPlanW<1024>; };
 
-// FP64 lines up to 256 points: radix-4 (and 2, 3) stages with 4 or 12
-// elements per thread.  An FP64 instruction occupies a sub-partition's FP64
-// unit for many cycles on this part, so a short line is transformed by more
-// threads with shorter per-thread chains; the extra stages cost shared
-// memory traffic, not FP64 work.
-template <int N> struct FftPlanD;
-HZ_PLAN_T(FftPlanD<8>, 8, 4, 4, 2)
-HZ_PLAN_T(FftPlanD<16>, 16, 4, 4, 4)
-HZ_PLAN_T(FftPlanD<24>, 24, 12, 4, 2, 3)
-HZ_PLAN_T(FftPlanD<32>, 32, 4, 4, 4, 2)
-HZ_PLAN_T(FftPlanD<64>, 64, 4, 4, 4, 4)
-HZ_PLAN_T(FftPlanD<96>, 96, 12, 4, 4, 2, 3)
-HZ_PLAN_T(FftPlanD<128>, 128, 4, 4, 4, 4, 2)
-HZ_PLAN_T(FftPlanD<192>, 192, 12, 4, 4, 4, 3)
-HZ_PLAN_T(FftPlanD<256>, 256, 4, 4, 4, 4, 4)
-#define HZ_DPLAN(NN)                                                       \
-  template <> struct RowPlan<double, NN> { using P = FftPlanD<NN>; };      \
-  template <> struct ColPlan<double, NN> { using P = FftPlanD<NN>; };
-HZ_DPLAN(8)
-HZ_DPLAN(16)
-HZ_DPLAN(24)
-HZ_DPLAN(32)
-HZ_DPLAN(64)
-HZ_DPLAN(96)
-HZ_DPLAN(128)
-HZ_DPLAN(192)
-HZ_DPLAN(256)
-#undef HZ_DPLAN
 #undef HZ_PLAN
 #undef HZ_PLAN_T
 

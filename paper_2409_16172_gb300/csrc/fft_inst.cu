@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "fft_int.cuh"
 #include "fft_kernels.cuh"
 
 #ifndef HZ_FFT_N
@@ -55,13 +56,74 @@ hz_status row_fwd_t(const double2* in, const double* scale, long rows_per_rhs, l
   return HZ_OK;
 }
 
+// complex128 passes (fft_int.cuh): blocks of full size, or of one line (a
+// quarter of the columns) where those would leave SMs without a block
+constexpr long kFew = 2 * 152;
+
+template <int LINES>
+hz_status irow_fwd_t(const double2* in, const double* scale, long rows, long nrhs, const int4* tw,
+                     double2* out, cudaStream_t st, const int* active) {
+  using B = IBlock<N, LINES, true>;
+  auto k = irow_fwd_kernel<N, LINES>;
+  HZ_TRY(smem_attr(k, B::SMEM));
+  HZ_CUDA(launch_pdl(k, dim3(unsigned((rows + LINES - 1) / LINES), unsigned(nrhs)), dim3(B::NT),
+                     B::SMEM, st, in, scale, rows, tw, out, active));
+  HZ_CUDA(cudaGetLastError());
+  return HZ_OK;
+}
+
 hz_status row_fwd(int prec, const double2* in, const double* scale, long rows_per_rhs, long nrows,
                   const void* tw, void* out, cudaStream_t st, const int* active, void* zero,
                   long zero_row_bytes) {
-  return prec == 0 ? row_fwd_t<double>(in, scale, rows_per_rhs, nrows, tw, out, st, active, zero,
-                                       zero_row_bytes)
-                   : row_fwd_t<float>(in, scale, rows_per_rhs, nrows, tw, out, st, active, zero,
-                                      zero_row_bytes);
+  if (prec == 0) {
+    // the complex128 x-inverse ends in a gather: nothing to clear
+    constexpr int L = ICfg<N>::ROWS;
+    const long nrhs = nrows / rows_per_rhs;
+    const bool few = (rows_per_rhs + L - 1) / L * nrhs < kFew;
+    return (few ? irow_fwd_t<1> : irow_fwd_t<L>)(in, scale, rows_per_rhs, nrhs,
+                                                 static_cast<const int4*>(tw),
+                                                 static_cast<double2*>(out), st, active);
+  }
+  return row_fwd_t<float>(in, scale, rows_per_rhs, nrows, tw, out, st, active, zero,
+                          zero_row_bytes);
+}
+
+template <int LINES>
+hz_status irow_inv_t(double2* planes, const unsigned long long* rowmask, int K, long rows,
+                     long nrhs, long n, const int4* tw, cudaStream_t st, const int* active) {
+  using B = IBlock<N, LINES, true>;
+  auto k = irow_inv_kernel<N, LINES>;
+  HZ_TRY(smem_attr(k, B::SMEM));
+  HZ_CUDA(launch_pdl(k, dim3(unsigned((rows + LINES - 1) / LINES), unsigned(K), unsigned(nrhs)),
+                     dim3(B::NT), B::SMEM, st, planes, rowmask, K, rows, n, tw, active));
+  HZ_CUDA(cudaGetLastError());
+  return HZ_OK;
+}
+
+// complex128: every (row, node) line in place, then the weighted gather
+hz_status row_inv_c128(const void* planes, const void* rec, const uchar2* segtab,
+                       const unsigned long long* rowmask, int K, long rows_per_rhs, long nrows,
+                       long n, double inv_n, const void* tw, void* out, cudaStream_t st,
+                       const int* active, const uchar4* gnode, const void* gw) {
+  constexpr int L = ICfg<N>::ROWS;
+  const long nrhs = nrows / rows_per_rhs;
+  const bool few = (rows_per_rhs + L - 1) / L * nrhs * K < kFew;
+  double2* pl = static_cast<double2*>(const_cast<void*>(planes));
+  HZ_TRY((few ? irow_inv_t<1> : irow_inv_t<L>)(pl, rowmask, K, rows_per_rhs, nrhs, n,
+                                               static_cast<const int4*>(tw), st, active));
+  const long total = nrows * N;
+  const long gblocks = std::min<long>((total + 255) / 256, 152L * 16);
+  if (gnode)
+    HZ_CUDA(launch_pdl(weighted_gather4_kernel<double, double2>, dim3(unsigned(gblocks)), dim3(256),
+                       0, st, pl, gnode, static_cast<const double2*>(gw), K, n, total, inv_n,
+                       static_cast<double2*>(out), active));
+  else
+    HZ_CUDA(launch_pdl(weighted_gather_kernel<double, double2>, dim3(unsigned(gblocks)), dim3(256),
+                       0, st, pl, static_cast<const double*>(rec), segtab, K, n, total, inv_n,
+                       static_cast<double2*>(out), active));
+  HZ_CUDA(cudaGetLastError());
+  count_launches(1);  // the phase counts one
+  return HZ_OK;
 }
 
 template <typename R, typename OutT>
@@ -111,11 +173,7 @@ hz_status row_inv_acc_t(const void* planes, const void* rec, const uchar2* segta
   }
   // fewer blocks of ROW_LINES rows than SMs: few rows
   const bool small = (nrows + C::ROW_LINES - 1) / C::ROW_LINES < 152L;
-  // the fused pass holds three E-element arrays per thread; complex128 with
-  // 30 elements per thread (lengths with a factor 5) would spill, so those
-  // take the in-place pass and the gather
-  constexpr bool fused_ok = !(sizeof(R) == 8 && C::RP::E > 16);
-  if (mode == 1 || (mode == 0 && small) || !fused_ok) {
+  if (mode == 1 || (mode == 0 && small)) {
     // few rows: (row, node) lines in parallel, in place, then the gather
     auto ki = row_inv_inplace_kernel<R, N, C::ROW_LINES>;
     HZ_TRY(smem_attr(ki, C::row_smem()));
@@ -133,18 +191,16 @@ hz_status row_inv_acc_t(const void* planes, const void* rec, const uchar2* segta
     count_launches(1);  // the phase counts one
     return HZ_OK;
   }
-  if constexpr (fused_ok) {
-    constexpr int lines = C::ROW_LINES;
-    auto k = row_inv_acc_kernel<R, N, OutT, C::ROW_LINES>;
-    HZ_TRY(smem_attr(k, C::row_acc_smem(lines)));
-    const long blocks = (nrows + lines - 1) / lines;
-    HZ_CUDA(launch_pdl(k, dim3(unsigned(blocks)), dim3(lines * C::TPL_ROW), C::row_acc_smem(lines),
-                       st, static_cast<const V*>(planes),
-                       static_cast<const typename RecT<R>::T*>(rec), segtab, nseg, rowmask, K,
-                       rows_per_rhs, nrows, n, R(inv_n), static_cast<const V*>(tw),
-                       static_cast<OutT*>(out), active));
-    HZ_CUDA(cudaGetLastError());
-  }
+  constexpr int lines = C::ROW_LINES;
+  auto k = row_inv_acc_kernel<R, N, OutT, C::ROW_LINES>;
+  HZ_TRY(smem_attr(k, C::row_acc_smem(lines)));
+  const long blocks = (nrows + lines - 1) / lines;
+  HZ_CUDA(launch_pdl(k, dim3(unsigned(blocks)), dim3(lines * C::TPL_ROW), C::row_acc_smem(lines),
+                     st, static_cast<const V*>(planes),
+                     static_cast<const typename RecT<R>::T*>(rec), segtab, nseg, rowmask, K,
+                     rows_per_rhs, nrows, n, R(inv_n), static_cast<const V*>(tw),
+                     static_cast<OutT*>(out), active));
+  HZ_CUDA(cudaGetLastError());
   return HZ_OK;
 }
 
@@ -155,8 +211,8 @@ hz_status row_inv_acc(int prec, int out_kind, const void* planes, const void* re
                       const unsigned long long* items, long nitems, const uchar4* gnode,
                       const void* gw) {
   if (prec == 0)
-    return row_inv_acc_t<double, double2>(planes, rec, segtab, nseg, rowmask, K, rows_per_rhs,
-                                          nrows, n, inv_n, tw, out, st, active, mode, items, nitems, gnode, gw);
+    return row_inv_c128(planes, rec, segtab, rowmask, K, rows_per_rhs, nrows, n, inv_n, tw, out, st,
+                        active, gnode, gw);
   if (out_kind == 0)
     return row_inv_acc_t<float, float2>(planes, rec, segtab, nseg, rowmask, K, rows_per_rhs,
                                         nrows, n, inv_n, tw, out, st, active, mode, items, nitems, gnode, gw);
@@ -181,12 +237,31 @@ hz_status line_pass_t(void* data, int nx, long outer, long S, long ostride, long
   return HZ_OK;
 }
 
+template <int SIGN, int TB>
+hz_status iline_t(double2* data, int nx, long outer, long S, long ostride, long bstride, int batch,
+                  const unsigned long long* omask, int K, const int4* tw, cudaStream_t st,
+                  const int* active, int per_rhs) {
+  using B = IBlock<N, TB, false>;
+  auto k = iline_kernel<N, SIGN, TB>;
+  HZ_TRY(smem_attr(k, B::SMEM));
+  const int ntile = (nx + TB - 1) / TB;
+  HZ_CUDA(launch_pdl(k, dim3(unsigned(ntile * outer), 1, unsigned(batch)), dim3(B::NT), B::SMEM, st,
+                     data, nx, ntile, S, ostride, bstride, omask, K, tw, active, per_rhs));
+  HZ_CUDA(cudaGetLastError());
+  return HZ_OK;
+}
+
 hz_status line_pass(int prec, int sign, void* data, int nx, long outer, long S, long ostride,
                     long bstride, int batch, const unsigned long long* omask, int K,
                     const void* tw, cudaStream_t st, const int* active, int per_rhs) {
-  if (prec == 0)
-    return sign < 0 ? line_pass_t<double, -1>(data, nx, outer, S, ostride, bstride, batch, omask, K, tw, st, active, per_rhs)
-                    : line_pass_t<double, +1>(data, nx, outer, S, ostride, bstride, batch, omask, K, tw, st, active, per_rhs);
+  if (prec == 0) {
+    constexpr int TB = ICfg<N>::TB, TF = ICfg<N>::TB_FEW;
+    const bool few = (nx + TB - 1) / TB * outer * batch < kFew;
+    auto go = sign < 0 ? (few ? iline_t<-1, TF> : iline_t<-1, TB>)
+                       : (few ? iline_t<+1, TF> : iline_t<+1, TB>);
+    return go(static_cast<double2*>(data), nx, outer, S, ostride, bstride, batch, omask, K,
+              static_cast<const int4*>(tw), st, active, per_rhs);
+  }
   return sign < 0 ? line_pass_t<float, -1>(data, nx, outer, S, ostride, bstride, batch, omask, K, tw, st, active, per_rhs)
                   : line_pass_t<float, +1>(data, nx, outer, S, ostride, bstride, batch, omask, K, tw, st, active, per_rhs);
 }
@@ -261,19 +336,42 @@ hz_status line_sym_inv_t(const void* vhat, void* planes, int nx, long outer, lon
   return HZ_OK;
 }
 
+template <int TB>
+hz_status isym_t(const void* vhat, void* planes, int nx, long outer, long S, long ostride, long n,
+                 int K, int batch, const void* xi2_x, const void* xi2_o, const void* xi2_l,
+                 const void* symA, const void* symG, const void* symD,
+                 const unsigned long long* smask, long smO, long smS, const void* tw,
+                 cudaStream_t st, const int* active) {
+  using B = IBlock<N, TB, false>;
+  auto k = symD ? isym_kernel<N, TB, true> : isym_kernel<N, TB, false>;
+  HZ_TRY(smem_attr(k, B::SMEM));
+  const int ntile = (nx + TB - 1) / TB;
+  HZ_CUDA(launch_pdl(k, dim3(unsigned(ntile * outer), unsigned(K), unsigned(batch)), dim3(B::NT),
+                     B::SMEM, st, static_cast<const double2*>(vhat), static_cast<double2*>(planes),
+                     nx, ntile, S, ostride, n, K, static_cast<const double*>(xi2_x),
+                     static_cast<const double*>(xi2_o), static_cast<const double*>(xi2_l),
+                     static_cast<const double2*>(symA), static_cast<const double2*>(symG),
+                     static_cast<const double*>(symD), smask, smO, smS,
+                     static_cast<const int4*>(tw), active));
+  HZ_CUDA(cudaGetLastError());
+  return HZ_OK;
+}
+
 hz_status line_sym_inv(int prec, const void* vhat, void* planes, int nx, long outer, long S,
                        long ostride, long n, int K, int batch, const void* xi2_x,
                        const void* xi2_o, const void* xi2_l, const void* symA, const void* symG,
                        const void* symD, const unsigned long long* smask, long smO, long smS,
                        const void* tw, const void* tw2, cudaStream_t st, const int* active,
                        int kpb, int pair) {
-  return prec == 0
-             ? line_sym_inv_t<double>(vhat, planes, nx, outer, S, ostride, n, K, batch, xi2_x,
-                                      xi2_o, xi2_l, symA, symG, symD, smask, smO, smS, tw, nullptr,
-                                      st, active, kpb, 0)
-             : line_sym_inv_t<float>(vhat, planes, nx, outer, S, ostride, n, K, batch, xi2_x,
-                                     xi2_o, xi2_l, symA, symG, symD, smask, smO, smS, tw, tw2, st,
-                                     active, kpb, pair);
+  if (prec == 0) {
+    constexpr int TB = ICfg<N>::TB, TF = ICfg<N>::TB_FEW;
+    const bool few = (nx + TB - 1) / TB * outer * K * batch < kFew;
+    return (few ? isym_t<TF> : isym_t<TB>)(vhat, planes, nx, outer, S, ostride, n, K, batch, xi2_x,
+                                           xi2_o, xi2_l, symA, symG, symD, smask, smO, smS, tw, st,
+                                           active);
+  }
+  return line_sym_inv_t<float>(vhat, planes, nx, outer, S, ostride, n, K, batch, xi2_x, xi2_o, xi2_l,
+                               symA, symG, symD, smask, smO, smS, tw, tw2, st, active, kpb, pair);
 }
 
 const FftOps ops = {N, row_fwd, row_inv_acc, line_pass, line_sym_inv};

@@ -69,7 +69,7 @@ bool fft_size_supported(int N);
 // Per-axis tables for one FFT length.
 struct AxisTables {
   int N = 0;
-  double2* tw64 = nullptr;  // exp(-2 pi i j / N)
+  int4* tw64 = nullptr;  // exp(-2 pi i j / N) times 2^61: (re, im) in limbs of 31 bits
   float2* tw32 = nullptr;
   float4* tw32p = nullptr;  // (re, re, im, im) of tw32, for paired lines
   double* xi2_64 = nullptr;  // squared wavenumber per bin

@@ -631,17 +631,25 @@ extern "C" hz_status hz_create_medium(const hz_grid* grid, const double* c, cons
     std::vector<double> xi;
     twiddles(N, tw);
     xi2_table(N, m->L, interp->symbol_kind, xi);
+    std::vector<int4> twi(N);  // times 2^61, in limbs of 31 bits (fft_int.cuh)
+    auto limbs = [](double v, int* hi, int* lo) {
+      const long long q = std::llrint(std::ldexp(v, 61));
+      *hi = int(q >> 31);
+      *lo = int(q & 0x7fffffff);
+    };
     std::vector<float2> twf(N);
     std::vector<float4> twp(N);
     std::vector<float> xif(N);
     for (int j = 0; j < N; ++j) {
+      limbs(tw[j].x, &twi[j].x, &twi[j].y);
+      limbs(tw[j].y, &twi[j].z, &twi[j].w);
       twf[j] = make_float2(float(tw[j].x), float(tw[j].y));
       twp[j] = make_float4(twf[j].x, twf[j].x, twf[j].y, twf[j].y);
       xif[j] = float(xi[j]);
     }
     AxisTables& t = m->ax[d];
     t.N = N;
-    if ((st = upload(m->arena, &t.tw64, tw, cs)) != HZ_OK) return fail(st);
+    if ((st = upload(m->arena, &t.tw64, twi, cs)) != HZ_OK) return fail(st);
     if ((st = upload(m->arena, &t.tw32, twf, cs)) != HZ_OK) return fail(st);
     if ((st = upload(m->arena, &t.tw32p, twp, cs)) != HZ_OK) return fail(st);
     if ((st = upload(m->arena, &t.xi2_64, xi, cs)) != HZ_OK) return fail(st);
