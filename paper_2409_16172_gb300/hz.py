@@ -192,9 +192,12 @@ def _dptr(a):
 
 
 def _stream(stream):
+    if stream is not None:
+        return _vp(stream.cuda_stream)
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return _vp(s.cuda_stream)
+    # the raw handle of torch.cuda.current_stream() without the Stream object,
+    # whose construction cost more than a small kernel's launch
+    return _vp(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _check_dev(x, name):
