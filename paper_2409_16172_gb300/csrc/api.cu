@@ -158,10 +158,46 @@ static hz_status ensure_planes(hz_plan* p, int prec) {
   return HZ_OK;
 }
 
+// Shape of the complex64 symbol pass for a last axis of N points and `points`
+// points over all right-hand sides, as (nodes per block, columns per thread).
+// Blocks of four nodes read the spectrum once for four planes and pay where
+// there are enough blocks without them (256^3 1393 -> 1257 us, 512^2 x 16
+// right-hand sides 266 -> 247, 2048^2 559 -> 509, 64^3 x 8 162 -> 149; but
+// 1024^2 104 -> 113, 128^3 163 -> 169).  A pair of columns needs the registers
+// of two lines: threads with 24 or 30 elements (factors 3 and 5) do better
+// with one column on small grids (192^2 20.8 -> 17.6 us, 360 x 480 41 -> 34,
+// 720^2 122 -> 111) and with half blocks or four nodes on large ones
+// (192^3 734 -> 674, 180^3 988 -> 750, 240^3 2520 -> 1902), except at 960,
+// 1440 and 2880 (1440^2 336 -> 369).
+static void sym_shape(int N, long points, int* kpb, int* pair) {
+  *kpb = 1;
+  *pair = 1;
+  if (N % 5 == 0) {
+    if (N <= 720 || N == 1920) {
+      *pair = 0;
+      if (N <= 720 && points >= (1l << 22)) *kpb = 4;
+    } else if (N == 2400 && points >= (1l << 22)) {
+      *kpb = 4;
+    }
+  } else if (N == 96 || N == 192) {
+    *pair = points < (1l << 17) ? 0 : 2;
+  } else if (points >= (1l << 21)) {
+    if (N == 256 || N == 512 || N == 2048) *kpb = 4;
+    if (N == 64) {
+      *kpb = 4;
+      *pair = 2;
+    }
+  }
+}
+
 // in: nrhs c128 vectors at stride n, each scaled by scale[b] (NULL = 1).
 // out_kind 0: c64 output, 1: c128 output.  prec 0: complex128 arithmetic.
+// by_size: untuned complex64 passes take their shape by size (applies); solves
+// keep one shape, because another rounding of the complex64 preconditioner
+// moves a solution by up to 1e-8 of its norm (1024^2, 100 Arnoldi steps).
 hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* scale, int nrhs,
-                        void* out, int out_kind, cudaStream_t st, const int* active) {
+                        void* out, int out_kind, cudaStream_t st, const int* active,
+                        bool by_size) {
   const hz_medium* m = p->med;
   HZ_TRY(ensure_planes(p, prec));
   const int nx = m->nx, ny = m->ny, nz = m->nz;
@@ -171,9 +207,12 @@ hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* s
   const AxisTables& tx = m->ax[0];
   const AxisTables& ty = m->ax[1];
   auto tw = [&](const AxisTables& t) -> const void* { return prec == 0 ? (const void*)t.tw64 : (const void*)t.tw32; };
-  // paired (two columns per thread) complex64 symbol pass unless tuned off
+  int kpb = 1, pair = 1;
+  if (by_size) sym_shape(m->dim == 2 ? ny : nz, n * p->max_nrhs, &kpb, &pair);
+  if (p->tune.syminv_kpb > 0) kpb = p->tune.syminv_kpb;
+  if (p->tune.col_pair >= 0) pair = p->tune.col_pair;
   auto tw2 = [&](const AxisTables& t) -> const void* {
-    return prec == 1 && p->tune.col_pair ? (const void*)t.tw32p : nullptr;
+    return prec == 1 && pair ? (const void*)t.tw32p : nullptr;
   };
   auto xi = [&](const AxisTables& t) -> const void* { return prec == 0 ? (const void*)t.xi2_64 : (const void*)t.xi2_32; };
   const void* A = prec == 0 ? (const void*)m->symA64 : (const void*)m->symA32;
@@ -186,8 +225,18 @@ hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* s
   const double rb = prec == 0 ? 8.0 : 4.0;          // interpolation record
   const double B = nrhs, K = m->K, dn = double(n);
   auto l2 = [](int N) { return std::log2(double(N)); };
+  // The x-inverse by size: up to 4096 rows one line per (row, node) fills the
+  // GPU best (256^2 18.7 -> 15.2 us, 720 x 960 113 -> 98, 1024^2 with K = 16
+  // 104 -> 96, 2048^2 559 -> 547; 512^2 x 16 right-hand sides, 8192 rows, 266
+  // -> 278).  Rows of one warp (512, 1024) need enough nodes per row for it
+  // (1024^2 with K = 8: 67 -> 70).  By the plan's right-hand sides, so that a
+  // result does not depend on how many a call has.
+  int mode = p->tune.rowinv_mode;
+  if (mode == 0 && by_size && prec == 1 && !m->generic && rows * p->max_nrhs <= 4096 &&
+      !((nx == 512 || nx == 1024) && m->rowk_used < 7.0 * double(rows)))
+    mode = 3;
   // the scattering x-inverse pass adds into out: cleared by the x-forward pass
-  const bool scatter = p->tune.rowinv_mode == 3;
+  const bool scatter = mode == 3 && prec == 1;
   {
     PhaseScope ps(st, PH_ROW_FWD, B * dn * (16.0 + s + (scatter ? so : 0.0)),
                   B * 5.0 * dn * l2(nx));
@@ -205,7 +254,7 @@ hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* s
                   B * K * (5.0 * dn * l2(ny) + 14.0 * dn));
     HZ_TRY(oy->line_sym_inv(prec, p->tmp, p->planes, nx, 1, nx, 0, n, m->K, nrhs, xi(tx), nullptr,
                             xi(ty), A, G, D, m->rowmask, 0, 1, tw(ty), tw2(ty), st, active,
-                            p->tune.syminv_kpb, p->tune.col_pair));
+                            kpb, pair));
   } else {
     const FftOps* oz = fft_ops(nz);
     const AxisTables& tz = m->ax[2];
@@ -220,7 +269,7 @@ hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* s
                     B * K * (5.0 * dn * l2(nz) + 14.0 * dn));
       HZ_TRY(oz->line_sym_inv(prec, p->tmp, p->planes, nx, ny, slab, nx, n, m->K, nrhs, xi(tx),
                               xi(ty), xi(tz), A, G, D, m->slabmask, 0, 1, tw(tz), tw2(tz), st,
-                              active, p->tune.syminv_kpb, p->tune.col_pair));
+                              active, kpb, pair));
     }
     {
       PhaseScope ps(st, PH_LINE, B * 2.0 * s * m->slabk_used * slab,
@@ -234,7 +283,7 @@ hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* s
                   B * (m->rowk_used * 5.0 * nx * l2(nx) + 8.0 * dn));
     HZ_TRY(ox->row_inv_acc(prec, out_kind, p->planes, rec, m->segtab, m->nseg, m->rowmask, m->K,
                            rows, rows * nrhs, n, 1.0 / double(n), tw(tx), out, st, active,
-                           p->tune.rowinv_mode, m->rowitems, m->nitems, m->gnode,
+                           mode, m->rowitems, m->nitems, m->gnode,
                            prec == 0 ? (const void*)m->gw64 : (const void*)m->gw32));
   }
   return HZ_OK;
@@ -361,5 +410,5 @@ extern "C" hz_status hz_apply_preconditioner(hz_plan* plan, const void* x, void*
   if (precision != 0 && precision != 1) return set_error(HZ_ERR_INVALID_ARG, "precision must be 0 or 1");
   HZ_TRY(check_device(plan->med));
   return precond_apply(plan, precision, static_cast<const double2*>(x), nullptr, nrhs, y, 1,
-                       static_cast<cudaStream_t>(stream), nullptr);
+                       static_cast<cudaStream_t>(stream), nullptr, true);
 }

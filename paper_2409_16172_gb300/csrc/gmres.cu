@@ -23,7 +23,8 @@
 
 namespace hz {
 hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* scale, int nrhs,
-                        void* out, int out_kind, cudaStream_t st, const int* active);
+                        void* out, int out_kind, cudaStream_t st, const int* active,
+                        bool by_size = false);
 }
 
 using namespace hz;

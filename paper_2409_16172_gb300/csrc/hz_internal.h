@@ -83,7 +83,9 @@ struct AxisTables {
 // global memory before it; launched with launch_pdl, a kernel's launch and
 // block scheduling then overlap the tail of the previous kernel (also as
 // programmatic edges inside captured graphs).  Without a PDL predecessor the
-// wait returns at once.
+// wait returns at once.  (Letting the next kernel launch as soon as this one
+// has started, griddepcontrol.launch_dependents up front, was measured: a
+// 256^2 apply 14 -> 22 us, a 128^2 solve 1.93 -> 2.97 ms.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
@@ -257,10 +259,10 @@ struct SolveWs;
 // choice): nodes per block of the last-axis symbol pass, form of the
 // x-inverse, columns per thread.
 struct Tune {
-  int syminv_kpb = 1;
+  int syminv_kpb = 0;   // 0: by size (sym_shape)
   int rowinv_mode = 0;  // FftOps::row_inv_acc mode (0..3)
-  int col_pair = 1;     // complex64 symbol pass: two columns per thread (2: in
-                        // half-size blocks)
+  int col_pair = -1;    // complex64 symbol pass: two columns per thread (2: in
+                        // half-size blocks); -1: by size
 };
 }
 

@@ -21,7 +21,8 @@
 
 namespace hz {
 hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* scale, int nrhs,
-                        void* out, int out_kind, cudaStream_t st, const int* active);
+                        void* out, int out_kind, cudaStream_t st, const int* active,
+                        bool by_size = false);
 }
 
 using namespace hz;
@@ -186,7 +187,6 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
       const float ms = tm.best_ms([&] {
         return precond_apply(p, prec, W, nullptr, B, out, prec == 1 ? 0 : 1, st, nullptr);
       });
-      if (kpb == def.syminv_kpb && pair == def.col_pair) tdef = ms;
       if (ms < tbest) {
         tbest = ms;
         best.syminv_kpb = kpb;
