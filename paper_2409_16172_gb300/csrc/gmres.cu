@@ -58,7 +58,6 @@ hz_status solve_ws_create(hz_plan* p) {
   A(w->ar.alloc(&ks.S1, size_t(B) * (m + 1)));
   A(w->ar.alloc(&ks.S2, size_t(B) * (m + 1)));
   A(w->ar.alloc(&ks.sigma, size_t(B) * (m + 1)));
-  A(w->ar.alloc(&ks.nrm2, B));
   A(w->ar.alloc(&ks.cs, size_t(B) * m));
   A(w->ar.alloc(&ks.sn, size_t(B) * m));
   A(w->ar.alloc(&ks.g, size_t(B) * (m + 1)));
@@ -351,13 +350,14 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
         HZ_TRY(launch_update_dots(Q, W, n, j, nrhs, ks.S1, m + 1, ks.sigma, B, ks.active, part,
                                   ks.S2, st));
       }
+      int nblk = 0;
       {
-        PhaseScope ps(st, PH_UPDATE, ub, fl + 4.0 * Bn, 2);
+        PhaseScope ps(st, PH_UPDATE, ub, fl + 4.0 * Bn);
         HZ_TRY(launch_update(Q, W, n, j, nrhs, ks.S2, m + 1, ks.sigma, B, ks.active, p->partial,
-                             ks.nrm2, j + 1 < m, st));
+                             &nblk, j + 1 < m, st));
       }
       PhaseScope ps(st, PH_GIVENS, 0.0, 0.0);
-      HZ_TRY(launch_givens(ks, j, nrhs, st));
+      HZ_TRY(launch_givens(ks, j, nrhs, p->partial, nblk, st));
       return HZ_OK;
     };
     if (p->opts.graphs && jmax == m && !history) {

@@ -15,7 +15,6 @@ struct KsDev {
   double2* S1;      // [b][m+1] first CGS sums
   double2* S2;      // [b][m+1] second CGS sums
   double* sigma;    // [i][b] scale of stored basis vector i
-  double* nrm2;     // [b] |w|^2 after the second pass
   double* cs;       // [b][m] rotation cosines
   double2* sn;      // [b][m] rotation sines
   double2* g;       // [b][m+1] rotated right-hand side
@@ -107,15 +106,16 @@ hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, in
                              const double2* S1, int ldS, const double* sigma, int ldsig,
                              const int* active, double2* partial, double2* S2,
                              cudaStream_t st);
-// w -= sum_i sigma_i^2 S_i V_i and |w|^2; keep: w also becomes V_{j+1}
+// w -= sum_i sigma_i^2 S_i V_i and nblk block sums of |w|^2 per right-hand
+// side; keep: w also becomes V_{j+1}
 hz_status launch_update(const Basis& Q, double2* w, long wstride, int j, int nrhs,
                         const double2* S, int ldS, const double* sigma, int ldsig,
-                        const int* active, double* partial, double* nrm2,
-                        bool keep, cudaStream_t st);
+                        const int* active, double* partial, int* nblk, bool keep, cudaStream_t st);
 // V_i = w
 hz_status launch_encode(const Basis& Q, const double2* w, long wstride, int i, int nrhs,
                         const int* active, cudaStream_t st);
-hz_status launch_givens(const KsDev& ks, int j, int nrhs, cudaStream_t st);
+hz_status launch_givens(const KsDev& ks, int j, int nrhs, const double* partial, int nblk,
+                        cudaStream_t st);
 hz_status launch_solution_update(int zprec, const void* Z, long ldb, double2* u, long ustride,
                                  long n, int nrhs, const double2* y, int ldy, const int* jn,
                                  cudaStream_t st);

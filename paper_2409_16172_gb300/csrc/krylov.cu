@@ -500,18 +500,30 @@ __device__ __forceinline__ double2 shfl_up_d2(double2 v, int o) {
   return make_double2(__shfl_up_sync(0xffffffffu, v.x, o), __shfl_up_sync(0xffffffffu, v.y, o));
 }
 
-// One warp per right-hand side: form column j of the Hessenberg matrix,
+constexpr int GT = 128;
+
+// One block per right-hand side: form column j of the Hessenberg matrix,
 // apply the earlier rotations, build the new one (c real, G [a;b] = [r;0]),
 // update g and the residual estimate, and retire converged / broken rows.
 // Applying rotations 0..j-1 is a linear recurrence on the running entry,
 //   x_0 = h_0,  x_{i+1} = -conj(s_i) x_i + c_i h_{i+1},  r_i = c_i x_i + s_i h_{i+1},
-// evaluated as a warp scan of affine maps (each lane composes a contiguous
+// evaluated by the first warp as a scan of affine maps (each lane composes a contiguous
 // chunk, a shuffle scan composes the chunks) instead of j serial steps.
-__global__ void givens_kernel(KsDev ks, int j, int nrhs) {
+// First |w|^2 from the update's nblk block sums (fixed order), by all warps.
+__global__ void __launch_bounds__(GT)
+givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
   pdl_wait();
   const int b = blockIdx.x;
+  if (!ks.active[b]) return;
+  __shared__ double nsum[GT / 32 + 1];
+  {
+    double v[1] = {0.0};
+    for (int i = threadIdx.x; i < nblk; i += GT) v[0] += partial[long(b) * nblk + i];
+    block_sum<1, GT>(v, nsum);
+  }
+  const double hn2 = nsum[GT / 32];  // |w|^2 after orthogonalisation
+  if (threadIdx.x >= 32) return;
   const int lane = threadIdx.x;
-  if (b >= nrhs || !ks.active[b]) return;
   const int m = ks.m;
   __shared__ double2 col[HZ_MAX_RESTART + 2];   // h, the new column before rotation
   __shared__ double2 rcol[HZ_MAX_RESTART + 2];  // rotated column
@@ -531,7 +543,6 @@ __global__ void givens_kernel(KsDev ks, int j, int nrhs) {
     hbits = max(hbits, max(absbits(h.x), absbits(h.y)));
     bad |= !isfinite(h.x) || !isfinite(h.y);
   }
-  const double hn2 = ks.nrm2[b];  // |w|^2 after orthogonalisation
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) hbits = max(hbits, __shfl_xor_sync(0xffffffffu, hbits, o));
   const double hmax = __longlong_as_double(hbits);
@@ -797,14 +808,12 @@ hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, in
 
 hz_status launch_update(const Basis& Q, double2* w, long wstride, int j, int nrhs,
                         const double2* S, int ldS, const double* sigma, int ldsig,
-                        const int* active, double* partial, double* nrm2,
-                        bool keep, cudaStream_t st) {
-  const int nblk = cgs_blocks(Q.ntiles, nrhs, 4);
-  HZ_TRY(launch_cgs<CG_UPDATE>(Q, nblk, CG_ROWS, w, wstride, j, nrhs, S, ldS, sigma, ldsig, active,
+                        const int* active, double* partial, int* nblk, bool keep, cudaStream_t st) {
+  *nblk = cgs_blocks(Q.ntiles, nrhs, 4);
+  HZ_TRY(launch_cgs<CG_UPDATE>(Q, *nblk, CG_ROWS, w, wstride, j, nrhs, S, ldS, sigma, ldsig, active,
                                reinterpret_cast<double2*>(partial),
                                keep ? Q.V + (j + 1) * Q.ldb * Q.n : nullptr,
                                keep ? Q.ev + (j + 1) * Q.ldb * Q.ntiles : nullptr, st));
-  HZ_CUDA(launch_pdl(reduce_r_kernel, dim3(unsigned(nrhs)), dim3(KT), 0, st, partial, nblk, nrm2));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
 }
@@ -817,8 +826,9 @@ hz_status launch_encode(const Basis& Q, const double2* w, long wstride, int i, i
   return HZ_OK;
 }
 
-hz_status launch_givens(const KsDev& ks, int j, int nrhs, cudaStream_t st) {
-  HZ_CUDA(launch_pdl(givens_kernel, dim3(nrhs), dim3(32), 0, st, ks, j, nrhs));
+hz_status launch_givens(const KsDev& ks, int j, int nrhs, const double* partial, int nblk,
+                        cudaStream_t st) {
+  HZ_CUDA(launch_pdl(givens_kernel, dim3(nrhs), dim3(GT), 0, st, ks, j, partial, nblk));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
 }

@@ -168,15 +168,20 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
                        m + 1, st);
   });
   r.upd_us = r.upd_us_default = 1e3f * tm.best_ms([&] {
-    return launch_update(Q, W, n, j, B, ks.S1, m + 1, ks.sigma, B, ks.active, p->partial, ks.nrm2,
+    int nblk = 0;
+    return launch_update(Q, W, n, j, B, ks.S1, m + 1, ks.sigma, B, ks.active, p->partial, &nblk,
                          false, st);
   });
 
   // symbol pass, through a whole preconditioner apply (its other passes do
   // not depend on the choice)
-  float tbest = 1e30f, tdef = 0.f;
+  float tbest = 1e30f;
   const int prec = p->opts.precision;
   void* out = p->Z;
+  p->tune = def;  // the untuned choice
+  const float tdef = tm.best_ms([&] {
+    return precond_apply(p, prec, W, nullptr, B, out, prec == 1 ? 0 : 1, st, nullptr);
+  });
   for (int pair : {1, 2, 0}) {
     if (pair != 1 && prec == 0) continue;  // FP64 has one form
     for (int kpb : {1, 2, 4}) {
