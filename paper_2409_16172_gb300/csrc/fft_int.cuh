@@ -518,14 +518,12 @@ isym_kernel(const double2* __restrict__ vhat, double2* __restrict__ planes, int 
   const double2* src = vhat + rhs * n + o * ostride + x0;
   const double2 A = symA[k], G = symG[k];
   const double D = HERM ? symD[k] : 0.0;
-  // a thread keeps its column (the block's columns divide its threads), so
-  // den = (A - G |xi|^2 of the other axes) - G |xi|^2 of this one
+  // a thread keeps its column (the block's columns divide its threads)
   static_assert(B::NT % TB == 0, "one column per thread");
   const int col = threadIdx.x % TB;
   const double sx = (col < have ? xi2_x[x0 + col] : 0.0) + (xi2_o ? xi2_o[o] : 0.0);
-  const double cx = fma(-G.x, sx, A.x), cy = fma(-G.y, sx, A.y);
-  const double cy2 = cy * cy;
   const bool real = G.y == 0.0;  // a real node: the imaginary part of den is constant
+  const double ay2 = A.y * A.y;
   unsigned hi = 0u;
 #pragma unroll 2
   for (int i = threadIdx.x; i < N * TB; i += B::NT) {
@@ -534,11 +532,12 @@ isym_kernel(const double2* __restrict__ vhat, double2* __restrict__ planes, int 
     if (col < have) {
       const double2 v = src[p * Si + col];
       // vhat q_k = vhat conj(den) / |den|^2,  den = A - G |xi|^2
-      const double sl = xi2_l[p];
-      const double dx = fma(-G.x, sl, cx);
-      double dy = cy, dy2 = cy2;
+      // (|xi|^2 rounded once before the cancellation near the resonance)
+      const double s2 = sx + xi2_l[p];
+      const double dx = fma(-G.x, s2, A.x);
+      double dy = A.y, dy2 = ay2;
       if (!real) {
-        dy = fma(-G.y, sl, cy);
+        dy = fma(-G.y, s2, A.y);
         dy2 = dy * dy;
       }
       const double inv = recip3(fma(dx, dx, dy2));
@@ -547,7 +546,7 @@ isym_kernel(const double2* __restrict__ vhat, double2* __restrict__ planes, int 
       r.y = fma(v.y, qx, -(v.x * qy));
       if (HERM && D != 0.0) {
         // derivative plane: vhat dq/dc = vhat q (D |xi|^2 q)
-        const double ds = D * (sx + sl), ux = qx * ds, uy = qy * ds;
+        const double ds = D * s2, ux = qx * ds, uy = qy * ds;
         r = make_double2(fma(r.x, ux, r.y * uy), fma(r.y, ux, -(r.x * uy)));
       }
     }
