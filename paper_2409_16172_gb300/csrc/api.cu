@@ -356,8 +356,8 @@ extern "C" hz_status hz_plan_create(hz_medium* med, const hz_solver_opts* opts, 
   const size_t evlen = size_t(B) * m * ((n + HZ_FX_TILE - 1) / HZ_FX_TILE);
   p->partial_len = std::max(budget - (evlen + 1) / 2,
                             size_t(m + 2) * 2 * HZ_CGS_BLOCKS * std::min(B, 4));
-  if ((st = p->arena.alloc(&p->partial, p->partial_len)) != HZ_OK) return fail(st);
-  if ((st = p->arena.alloc(&p->ev, evlen)) != HZ_OK) return fail(st);
+  if ((st = p->arena.alloc(&p->partial, p->partial_len + (evlen + 1) / 2)) != HZ_OK) return fail(st);
+  p->ev = reinterpret_cast<int*>(p->partial + p->partial_len);
   *out = p;
   return HZ_OK;
 }

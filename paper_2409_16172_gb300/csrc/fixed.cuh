@@ -5,11 +5,12 @@
 // (32 x 32 + 64 bits).  Sums of products over FP64 vectors are therefore made
 // in integers: a tile of FX_TILE consecutive points shares one binary
 // exponent E (the largest of its real and imaginary parts), a value is the
-// integer v = x 2^(FX_TOP + 1023 - E) rounded to nearest, |v| <= 2^54, held
-// as two signed limbs v = hi 2^28 + lo, |hi| <= 2^26, |lo| <= 2^27.  A value
-// within a factor 2 of the tile's largest keeps all 53 bits; a smaller one is
-// exact to 2^-54 of the tile's largest, half an ulp of that value.  The four
-// limb products are exact and are added exactly in 64 bits.
+// integer v = x 2^(FX_TOP + 1023 - E) rounded to nearest, |v| <= 2^54, held as
+// two limbs v = hi 2^27 + lo.  A value within a factor 2 of the tile's largest
+// keeps all 53 bits; a smaller one is exact to 2^-54 of the tile's largest,
+// half an ulp of that value.  The limb products hi hi and hi lo are exact and
+// are added exactly in 64 bits; lo lo, at most 2^-55 of the largest product
+// and of mean zero, is left out (one factor's lo is symmetric about zero).
 #pragma once
 #include "hz_internal.h"
 
@@ -21,44 +22,49 @@ constexpr int FX_TOP = 53;           // bit of the leading one of a value with e
 __device__ __forceinline__ int fx_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 __device__ __forceinline__ int fx_exp(double2 z) { return max(fx_exp(z.x), fx_exp(z.y)); }
 
-// x 2^(FX_TOP + 1023 - E) to the nearest integer, E >= exponent of x; integer
-// operations only.  Subnormals count as zero.
+// the smallest E that tiles use: zeros and subnormals then shift out
+constexpr int FX_EMIN = 64;
+
+// x 2^(FX_TOP + 1023 - E) to the nearest integer, E >= exponent of x and
+// E >= FX_EMIN; integer operations only.  Subnormals count as zero.
 __device__ __forceinline__ long long fx_from(double x, int E) {
   const int hi = __double2hiint(x);
-  const int ex = (hi >> 20) & 0x7ff;
-  const int sh = E - ex;
-  const unsigned long long m =
-      (static_cast<unsigned long long>((hi & 0xfffff) | 0x100000) << 32) | unsigned(__double2loint(x));
-  const int s = 9 + sh;  // m << 10 has its leading one at bit 62
-  const unsigned long long v = ((m << 10) + (1ull << ((s - 1) & 63))) >> (s & 63);
+  const unsigned lo = unsigned(__double2loint(x));
+  const int sh = E - ((hi >> 20) & 0x7ff);
+  const unsigned mh = unsigned((hi & 0xfffff) | 0x100000);
+  unsigned long long t = static_cast<unsigned long long>(__funnelshift_l(lo, mh, 2)) << 32 | (lo << 2);
+  asm("shr.u64 %0, %0, %1;" : "+l"(t) : "r"(sh));  // zero past 63
+  const long long v = static_cast<long long>((t + 1) >> 1);
   const long long sg = hi >> 31;
-  return (ex == 0 || s > 63) ? 0ll : ((static_cast<long long>(v) ^ sg) - sg);
+  return (v ^ sg) - sg;
 }
 
-// limbs of v: low 28 bits with sign, and the rest
-__device__ __forceinline__ int fx_lo(long long v) { return int(unsigned(v) << 4) >> 4; }
-__device__ __forceinline__ int fx_hi(long long v) { return int((v + (1ll << 27)) >> 28); }
-
+// limbs of v: with lo symmetric, |lo| <= 2^26, |hi| <= 2^27
+__device__ __forceinline__ int fx_lo(long long v) { return int(unsigned(v) << 5) >> 5; }
+__device__ __forceinline__ int fx_hi(long long v) { return int((v + (1ll << 26)) >> 27); }
 // a complex value as (re hi, re lo, im hi, im lo)
 __device__ __forceinline__ int4 fx_pack(double2 z, int E) {
   const long long a = fx_from(z.x, E), b = fx_from(z.y, E);
   return make_int4(fx_hi(a), fx_lo(a), fx_hi(b), fx_lo(b));
+}
+// the same with 0 <= lo < 2^27 (the other factor's lo is symmetric)
+__device__ __forceinline__ int4 fx_pack_floor(double2 z, int E) {
+  const long long a = fx_from(z.x, E), b = fx_from(z.y, E);
+  return make_int4(int(a >> 27), int(unsigned(a) & 0x7ffffffu), int(b >> 27),
+                   int(unsigned(b) & 0x7ffffffu));
 }
 
 __device__ __forceinline__ long long mad_w(int a, int b, long long c) {
   return static_cast<long long>(a) * b + c;
 }
 
-// hh 2^56 + x 2^28 + ll in units of 2^(56 - SH), rounded to nearest
-template <int SH>
-__device__ __forceinline__ long long fx_sum(long long hh, long long x, long long ll) {
-  const long long y = x + ((ll + (1ll << 27)) >> 28);
-  return (hh << SH) + ((y + (1ll << (27 - SH))) >> (28 - SH));
+// hh 2^54 + x 2^27 in units of 2^54, rounded to nearest
+__device__ __forceinline__ long long fx_sum(long long hh, long long x) {
+  return hh + ((x + (1ll << 26)) >> 27);
 }
-// fx_to's k for fx_sum<SH> of products of values whose (biased) exponents add
-// up to E
-template <int SH>
-__device__ __forceinline__ int fx_unit(int E) { return E + 56 - SH - 2 * FX_TOP - 2 * 1023; }
+// fx_to's k for fx_sum of products of values whose (biased) exponents add up
+// to E
+__device__ __forceinline__ int fx_unit(int E) { return E + 54 - 2 * FX_TOP - 2 * 1023; }
 
 // t 2^k; a result below the normal range is zero
 __device__ __forceinline__ double fx_to(long long t, int k) {

@@ -49,16 +49,16 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
 // ---------------------------------------------------------------------------
 // Gram-Schmidt kernels over the basis in block fixed-point form (fixed.cuh).
 //
-// What bounds them: past about 16 vectors the basis in HBM, 16 bytes a point
-// and vector, before that the work per tile (w to and from integers, folding
-// the sums).  2^24 points: dots 5.4 TB/s of basis at j = 20 and 5.9 at
-// j = 39, update 5.1 and 5.4; in FP64 the same sums were bound by the FP64
-// pipe at 2.1-2.5 TB/s.  A 256^3 Arnoldi step spends 3.7 ms here instead of
-// 9.2.  A
-// block takes one tile of FX_TILE points at a time.  Its basis rows (one row:
-// the tile's 128 points of one vector, 2 KB) come through shared memory by
-// cp.async, so that the loads in flight do not cost registers and run ahead
-// over tile boundaries.
+// What bounds them: past about 16 vectors dots and update run at the basis in
+// HBM, 16 bytes a point and vector; before that, and in the kernel that does
+// both, at the latency of the tile's phases with 8 to 16 warps per SM.  2^24
+// points: dots 6.0 TB/s of basis at j = 20 and 39, update 4.9 and 5.4, update
+// and dots in one 1.59 and 3.29 ms; in FP64 the same sums were bound by the
+// FP64 pipe at 2.1-2.5 TB/s.  A 256^3 Arnoldi step (j = 17 on average) spends
+// 3.2 ms here instead of 9.2.  A block takes one tile of FX_TILE points at a
+// time.  Its basis rows (one row: the tile's 128 points of one vector, 2 KB)
+// come through shared memory by cp.async, so that the loads in flight do not
+// cost registers and run ahead over tile boundaries.
 //   update side  a thread owns a point and runs over the vectors
 //   dot side     the vectors are dealt to the half warps; a lane takes CG_U
 //                points, and the integer sums of CG_NB vectors are folded
@@ -80,8 +80,8 @@ constexpr int CG_ROWS = 24;               // ring rows when rows only pass throu
 constexpr int CG_DEPTH = CG_ROWS / CG_HALVES;  // dot side: rows in flight per half warp
 constexpr int CG_NU = 4;                       // update side: rows per copy group
 constexpr int CG_GROUPS = CG_ROWS / CG_NU;     // and groups in flight
-constexpr int CG_MAXROWS = 34;            // ring rows at most (three blocks per SM)
-constexpr int CG_FUSED = 22;              // vectors at most in CG_UPDATE_DOTS
+constexpr int CG_MAXROWS = 52;            // ring rows at most (two blocks per SM)
+constexpr int CG_FUSED = 44;              // vectors at most in CG_UPDATE_DOTS
 constexpr size_t CG_ROW_BYTES = FX_TILE * sizeof(int4);
 
 __device__ __forceinline__ void copy16(int4* dst, const int4* src) {
@@ -120,39 +120,49 @@ __device__ __forceinline__ int max_of(const int* red) {
   return r;
 }
 
-// exact limb sums of conj(v) y (re, and the two halves of im)
+// a coefficient against the exponent E >= its own; one of a zero (or
+// subnormal) part, which fx_from's E may not be too small for, by itself
+__device__ __forceinline__ int4 coef_limbs(double2 c, int E) {
+  int4 r = fx_pack(c, E);
+  if (fx_exp(c.x) == 0) r.x = r.y = 0;
+  if (fx_exp(c.y) == 0) r.z = r.w = 0;
+  return r;
+}
+
+// limb sums of conj(v) y (re, and the two halves of im)
 struct DotAcc {
-  long long rh = 0, rx = 0, rl = 0, ph = 0, px = 0, pl = 0, qh = 0, qx = 0, ql = 0;
+  long long rh = 0, rx = 0, ph = 0, px = 0, qh = 0, qx = 0;
   __device__ __forceinline__ void add(const int4& v, const int4& y) {
     rh = mad_w(v.z, y.z, mad_w(v.x, y.x, rh));
-    rx = mad_w(v.z, y.w, mad_w(v.w, y.z, mad_w(v.x, y.y, mad_w(v.y, y.x, rx))));
-    rl = mad_w(v.w, y.w, mad_w(v.y, y.y, rl));
     ph = mad_w(v.x, y.z, ph);
-    px = mad_w(v.x, y.w, mad_w(v.y, y.z, px));
-    pl = mad_w(v.y, y.w, pl);
     qh = mad_w(v.z, y.x, qh);
+    rx = mad_w(v.z, y.w, mad_w(v.w, y.z, mad_w(v.x, y.y, mad_w(v.y, y.x, rx))));
+    px = mad_w(v.x, y.w, mad_w(v.y, y.z, px));
     qx = mad_w(v.z, y.y, mad_w(v.w, y.x, qx));
-    ql = mad_w(v.w, y.y, ql);
   }
-  // |hh| <= 2^57 over a lane's CG_U points: the sum over 16 lanes fits
-  __device__ __forceinline__ long long re() const { return fx_sum<1>(rh, rx, rl); }
-  __device__ __forceinline__ long long im() const { return fx_sum<1>(ph - qh, px - qx, pl - ql); }
+  // |hh| <= 2^58 over a lane's CG_U points: the sum over 16 lanes fits
+  __device__ __forceinline__ long long re() const { return fx_sum(rh, rx); }
+  __device__ __forceinline__ long long im() const { return fx_sum(ph - qh, px - qx); }
 };
-// exact limb sums of c v
+// limb sums of c v
 struct UpdAcc {
-  long long rh = 0, rx = 0, rl = 0, ih = 0, ix = 0, il = 0;
+  long long rh = 0, rx = 0, ih = 0, ix = 0;
   __device__ __forceinline__ void add(const int4& c, const int4& v) {
     const int nh = -c.z, nl = -c.w;
     rh = mad_w(nh, v.z, mad_w(c.x, v.x, rh));
-    rx = mad_w(nh, v.w, mad_w(nl, v.z, mad_w(c.x, v.y, mad_w(c.y, v.x, rx))));
-    rl = mad_w(nl, v.w, mad_w(c.y, v.y, rl));
     ih = mad_w(c.z, v.x, mad_w(c.x, v.z, ih));
+    rx = mad_w(nh, v.w, mad_w(nl, v.z, mad_w(c.x, v.y, mad_w(c.y, v.x, rx))));
     ix = mad_w(c.z, v.y, mad_w(c.w, v.x, mad_w(c.x, v.w, mad_w(c.y, v.z, ix))));
-    il = mad_w(c.w, v.y, mad_w(c.y, v.w, il));
   }
-  // |hh| <= 2^60 over HZ_MAX_RESTART + 1 vectors
-  __device__ __forceinline__ long long re() const { return fx_sum<2>(rh, rx, rl); }
-  __device__ __forceinline__ long long im() const { return fx_sum<2>(ih, ix, il); }
+  __device__ __forceinline__ void join(const UpdAcc& o) {
+    rh += o.rh;
+    rx += o.rx;
+    ih += o.ih;
+    ix += o.ix;
+  }
+  // |hh| <= 2 (HZ_MAX_RESTART + 1) 2^54 < 2^63
+  __device__ __forceinline__ long long re() const { return fx_sum(rh, rx); }
+  __device__ __forceinline__ long long im() const { return fx_sum(ih, ix); }
 };
 
 template <int MODE>
@@ -252,29 +262,31 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
     copy_commit();
     qs = qs + 1 == CG_GROUPS ? 0 : qs + 1;
   };
-  // CG_UPDATE_DOTS: all rows of a tile stay until its dots are done; row i of
-  // the block's k-th tile is at ring row (k (j+1) + i) mod rows
-  auto copy_part = [&](long t, int base, int lo, int hi) {  // rows lo <= i < hi of tile t
+  // CG_UPDATE_DOTS: all rows of a tile stay until its dots are done.  Row i of
+  // the block's even tiles is at ring row i, of its odd ones at rows - 1 - i:
+  // the first rows - (j + 1) rows of the next tile never meet this one's.
+  auto ring_row = [&](bool odd, int i) { return ring + (odd ? rows - 1 - i : i) * FX_TILE; };
+  auto copy_part = [&](long t, bool odd, int lo, int hi) {  // rows lo <= i < hi of tile t
     const long p = t * FX_TILE + tid;
     if (t < ntiles && p < n) {
-      int r = base + lo;
-      r = r >= rows ? r - rows : r;
+      int4* d = ring_row(odd, lo) + tid;
+      const int step = odd ? -FX_TILE : FX_TILE;
       const int4* s = Vb + lo * vs + p;
 #pragma unroll 4
       for (int i = lo; i < hi; ++i) {
-        copy16(ring + r * FX_TILE + tid, s);
+        copy16(d, s);
         s += vs;
-        r = r + 1 == rows ? 0 : r + 1;
+        d += step;
       }
     }
     copy_commit();
   };
-  int base = 0;
+  bool odd = false;
   const int ahead = MODE == CG_UPDATE_DOTS ? min(j + 1, rows - (j + 1)) : 0;
   if (MODE == CG_DOTS) {
     for (int k = 0; k < CG_DEPTH; ++k) copy_row();
   } else if (MODE == CG_UPDATE_DOTS) {
-    copy_part(tile, base, 0, ahead);
+    copy_part(tile, odd, 0, ahead);
   } else {
     for (int k = 0; k < CG_GROUPS; ++k) copy_group();
   }
@@ -287,7 +299,7 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
     warp_max(tid <= j ? ec + e0 : 0, redF);
     __syncthreads();
     F = max_of(redF);
-    if (tid <= j) cl[tid] = fx_pack(ci, F - e0);
+    if (tid <= j) cl[tid] = coef_limbs(ci, F - e0);
     __syncthreads();
   }
 
@@ -299,26 +311,30 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
     xn = load_w(tile + dt);
     const int e1 = tile_exp(tile + dt);
     if (UPD) {
-      UpdAcc a;
+      UpdAcc a, a2;  // alternate rows: shorter chains
       if (MODE == CG_UPDATE_DOTS) {
         // the rest of this tile's rows, and what fits of the next tile's
-        copy_part(tile, base, ahead, j + 1);
-        int nb = base + j + 1;
-        nb = nb >= rows ? nb - rows : nb;
-        copy_part(tile + dt, nb, 0, ahead);
+        copy_part(tile, odd, ahead, j + 1);
+        copy_part(tile + dt, !odd, 0, ahead);
+        const int4* s = ring_row(odd, 0) + tid;
+        const int step = odd ? -FX_TILE : FX_TILE;
+        auto rows_of = [&](int lo, int hi) {
+          int i = lo;
+#pragma unroll 2
+          for (; i + 2 <= hi; i += 2) {
+            a.add(cl[i], s[0]);
+            a2.add(cl[i + 1], s[step]);
+            s += 2 * step;
+          }
+          if (i < hi) {
+            a.add(cl[i], s[0]);
+            s += step;
+          }
+        };
         copy_wait<2>();
-        int r = base;
-#pragma unroll 2
-        for (int i = 0; i < ahead; ++i) {
-          a.add(cl[i], ring[r * FX_TILE + tid]);
-          r = r + 1 == rows ? 0 : r + 1;
-        }
+        rows_of(0, ahead);
         copy_wait<1>();
-#pragma unroll 2
-        for (int i = ahead; i <= j; ++i) {
-          a.add(cl[i], ring[r * FX_TILE + tid]);
-          r = r + 1 == rows ? 0 : r + 1;
-        }
+        rows_of(ahead, j + 1);
       } else {
         for (int k = 0; k < ng; ++k) {
           copy_wait<CG_GROUPS - 1>();
@@ -326,17 +342,18 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
           const int4* s = ring + rs * CG_NU * FX_TILE + tid;
           if (i0 + CG_NU <= j + 1) {
 #pragma unroll
-            for (int u = 0; u < CG_NU; ++u) a.add(cl[i0 + u], s[u * FX_TILE]);
+            for (int u = 0; u < CG_NU; ++u) (u & 1 ? a2 : a).add(cl[i0 + u], s[u * FX_TILE]);
           } else {
 #pragma unroll
             for (int u = 0; u < CG_NU; ++u)
-              if (i0 + u <= j) a.add(cl[i0 + u], s[u * FX_TILE]);
+              if (i0 + u <= j) (u & 1 ? a2 : a).add(cl[i0 + u], s[u * FX_TILE]);
           }
           copy_group();
           rs = rs + 1 == CG_GROUPS ? 0 : rs + 1;
         }
       }
-      const int k = fx_unit<2>(F);
+      a.join(a2);
+      const int k = fx_unit(F);
       const double dr = fx_to(a.re(), k), di = fx_to(a.im(), k);
       x = MODE == CG_COMBINE ? make_double2(dr, di) : make_double2(x.x - dr, x.y - di);
       if (in) wb[p] = x;
@@ -348,14 +365,14 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
     __syncthreads();
     if (UPD) {
       F = max_of(redF);
-      if (tid <= j) cl[tid] = fx_pack(ci, F - e1);
+      if (tid <= j) cl[tid] = coef_limbs(ci, F - e1);
     }
-    const int E = MODE != CG_COMBINE ? max_of(redw) : 0;
+    const int E = MODE != CG_COMBINE ? max(max_of(redw), FX_EMIN) : 0;
     if (MODE == CG_UPDATE && Vnew) {
       if (in) Vnew[long(b) * n + p] = fx_pack(x, E);
       if (tid == 0) enew[long(b) * ntiles + tile] = E;
     }
-    if (DOT) wl[tid] = fx_pack(x, E);
+    if (DOT) wl[tid] = fx_pack_floor(x, E);
     __syncthreads();
     if (DOT) {
       int4 wr[CG_U];
@@ -374,8 +391,8 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
               copy_wait<CG_DEPTH - 1>();
               r = hw * CG_DEPTH + rs;
             } else {
-              r = base + min(i0 + (hw & 1) + CG_HALVES * c, j);
-              r = r >= rows ? r - rows : r;
+              r = min(i0 + (hw & 1) + CG_HALVES * c, j);
+              if (odd) r = rows - 1 - r;
             }
             const int4* s = ring + r * FX_TILE + hl;
             DotAcc a;
@@ -392,7 +409,7 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
         }
         const long long sr = fold4(tr, lane), si = fold4(ti, lane);
         if ((lane & 3) == 0 && is <= j) {
-          const int k = fx_unit<1>(E + e);
+          const int k = fx_unit(E + e);
           double2 s = sacc[is];
           s.x += fx_to(sr, k);
           s.y += fx_to(si, k);
@@ -400,8 +417,7 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
         }
       }
       if (MODE == CG_UPDATE_DOTS) {
-        base += j + 1;
-        base = base >= rows ? base - rows : base;
+        odd = !odd;
         __syncthreads();  // the tile's rows are free
       }
     }
@@ -432,7 +448,7 @@ encode_kernel(const double2* __restrict__ w, long wstride, long n, long ntiles,
   const double2 x = p < n ? w[b * wstride + p] : make_double2(0.0, 0.0);
   warp_max(fx_exp(x), red);
   __syncthreads();
-  const int E = max_of(red);
+  const int E = max(max_of(red), FX_EMIN);
   if (p < n) V[long(b) * n + p] = fx_pack(x, E);
   if (threadIdx.x == 0) ev[long(b) * ntiles + blockIdx.x] = E;
 }
@@ -786,17 +802,17 @@ hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, in
                              const double2* S1, int ldS, const double* sigma, int ldsig,
                              const int* active, double2* partial, double2* S2,
                              cudaStream_t st) {
-  // One kernel while a tile's rows and part of the next tile's fit the shared
-  // memory of a third of an SM; past that its few warps cost more than the
-  // second read of the basis (2^24 points: j = 9 1112 us against 1238 us in
-  // two kernels, j = 20 2104 against 2153, j = 39 4203 against 3806).
+  // One kernel while a tile's rows fit the shared memory of half an SM, with as
+  // many blocks per SM as hold them: what it lacks is warps, not room for the
+  // next tile's rows (2^24 points, j = 22: four blocks of 24 rows 1703 us, three
+  // of 34 1727, two of 52 2001, two kernels 2270; j = 39: 3290 against 3780).
   if (j + 1 > CG_FUSED) {
     HZ_TRY(launch_cgs<CG_UPDATE>(Q, cgs_blocks(Q.ntiles, nrhs, 4), CG_ROWS, w, wstride, j, nrhs,
                                  S1, ldS, sigma, ldsig, active, partial, nullptr, nullptr, st));
     return launch_dots(Q, w, wstride, j, nrhs, active, partial, S2, ldS, st);
   }
-  const int per_sm = j + 1 <= 16 ? 4 : 3;
-  const int rows = per_sm == 4 ? CG_ROWS : CG_MAXROWS;
+  const int per_sm = j + 1 <= CG_ROWS ? 4 : (j + 1 <= 34 ? 3 : 2);
+  const int rows = per_sm == 4 ? CG_ROWS : (per_sm == 3 ? 34 : CG_MAXROWS);
   const int nblk = cgs_blocks(Q.ntiles, nrhs, per_sm);
   HZ_TRY(launch_cgs<CG_UPDATE_DOTS>(Q, nblk, rows, w, wstride, j, nrhs, S1, ldS, sigma, ldsig,
                                     active, partial, nullptr, nullptr, st));

@@ -2,8 +2,9 @@
 of one unpreconditioned Arnoldi cycle against an Arnoldi process (CGS2, FP64)
 written here with the oracle's operator, at sizes around the kernels' edges:
 grids of less than one tile of 128 points, of whole tiles and of a tile and a
-bit, cycles on both sides of the fused kernel's limit of 22 vectors and of its
-ring's 16, one to 128 vectors, several right-hand sides of very different size."""
+bit, cycles across the fused kernel's ring sizes (24, 34 and 52 rows) and its
+limit of 44 vectors, one to 128 vectors, several right-hand sides of very
+different size."""
 import numpy as np
 import pytest
 
@@ -18,8 +19,8 @@ pytestmark = pytest.mark.gpu
 # entry when f is perturbed by 1e-15 relative (four perturbations each, the
 # NumPy process below): rounding of a few 1e-16 per operation stays far below
 TOL = 1e-12
-CASES = [((8, 8), 1, 1), ((8, 8), 6, 2), ((12, 12), 16, 1), ((16, 24), 17, 3), ((24, 20), 22, 1),
-         ((24, 20), 23, 2), ((8, 12, 16), 40, 1), ((48, 64), 64, 1), ((64, 96), 128, 2)]
+CASES = [((8, 8), 1, 1), ((8, 8), 6, 2), ((12, 12), 16, 1), ((16, 24), 17, 3), ((24, 20), 24, 1),
+         ((24, 20), 25, 2), ((8, 12, 16), 36, 1), ((48, 48), 46, 1), ((48, 64), 64, 1), ((64, 96), 128, 2)]
 
 
 def arnoldi(apply_op, f, m):
