@@ -266,7 +266,11 @@ template <int N_, int LINES_, bool ROWS> struct IBlock {
   static constexpr bool BY_ROWS = ROWS;
   static constexpr int PADN = N + N / 8 + 1;
   static constexpr int want() {
-    int t = (N * LINES / 9 + 31) / 32 * 32;
+    // about one butterfly per thread; small blocks more threads, so that the
+    // FP64 parts spread over an SM's four units
+    const int points = N * LINES;
+    int t = (points / (points <= 512 ? 2 : 9) + 31) / 32 * 32;
+    if (points <= 512 && t > 128) t = 128;
     return t < 32 ? 32 : (t > 256 ? 256 : t);
   }
   static constexpr int NT = want();
