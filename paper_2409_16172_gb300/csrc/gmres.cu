@@ -31,6 +31,8 @@ using namespace hz;
 
 namespace {
 
+constexpr int kDirectCycles = 3;  // full cycles of a plan before one is captured
+
 bool is_device_ptr(const void* ptr) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
@@ -360,10 +362,15 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
       HZ_TRY(launch_givens(ks, j, nrhs, p->partial, nblk, st));
       return HZ_OK;
     };
-    if (p->opts.graphs && jmax == m && !history) {
+    const bool full = p->opts.graphs && jmax == m && !history;
+    if (full && (w.cyc_exec || ++w.cyc_direct > kDirectCycles)) {
       // The whole cycle as one CUDA graph, captured once per plan and right-
       // hand-side count and replayed; steps after a right-hand side retires
-      // return at once on its device-side flag.
+      // return at once on its device-side flag.  Capturing costs about four
+      // times what a replay saves over direct launches (128^2, 30 steps: 1.1 ms
+      // against 0.3 ms), so a plan's first cycles run directly: a served
+      // request on its own plan is done after a few (four requests of 256^2:
+      // 18.7 -> 11.0 ms).
       // captured on and replayed from the plan's own stream (the legacy
       // default stream cannot be captured), ordered after / before st
       if (!w.gstream) HZ_CUDA(cudaStreamCreateWithFlags(&w.gstream, cudaStreamNonBlocking));

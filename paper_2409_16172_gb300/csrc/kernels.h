@@ -39,6 +39,7 @@ struct SolveWs {
   cudaEvent_t t0 = nullptr, t1 = nullptr;
   cudaGraphExec_t cyc_exec = nullptr;  // captured Arnoldi cycle (opts.graphs)
   int cyc_nrhs = 0, cyc_kernels = 0;
+  int cyc_direct = 0;                  // full cycles run without a graph
   cudaStream_t gstream = nullptr;      // stream the cycle graph is captured on / replayed from
   cudaEvent_t gev[2] = {nullptr, nullptr};
 };
