@@ -53,7 +53,7 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
 // HBM, 16 bytes a point and vector; before that, and in the kernel that does
 // both, at the latency of the tile's phases with 8 to 16 warps per SM.  2^24
 // points: dots 6.0 TB/s of basis at j = 20 and 39, update 4.9 and 5.4, update
-// and dots in one 1.59 and 3.29 ms; in FP64 the same sums were bound by the
+// and dots in one 1.52 and 3.05 ms; in FP64 the same sums were bound by the
 // FP64 pipe at 2.1-2.5 TB/s.  A 256^3 Arnoldi step (j = 17 on average) spends
 // 3.2 ms here instead of 9.2.  A block takes one tile of FX_TILE points at a
 // time.  Its basis rows (one row: the tile's 128 points of one vector, 2 KB)
@@ -129,19 +129,26 @@ __device__ __forceinline__ int4 coef_limbs(double2 c, int E) {
   return r;
 }
 
-// limb sums of conj(v) y (re, and the two halves of im)
+// limb sums of conj(v) y (re, and the two halves of im); no sum takes more
+// than two products of a point, so that none is a long chain
 struct DotAcc {
-  long long rh = 0, rx = 0, ph = 0, px = 0, qh = 0, qx = 0;
+  long long rh = 0, rx = 0, ry = 0, ph = 0, px = 0, qh = 0, qx = 0;
   __device__ __forceinline__ void add(const int4& v, const int4& y) {
-    rh = mad_w(v.z, y.z, mad_w(v.x, y.x, rh));
+    rh = mad_w(v.x, y.x, rh);
     ph = mad_w(v.x, y.z, ph);
     qh = mad_w(v.z, y.x, qh);
-    rx = mad_w(v.z, y.w, mad_w(v.w, y.z, mad_w(v.x, y.y, mad_w(v.y, y.x, rx))));
-    px = mad_w(v.x, y.w, mad_w(v.y, y.z, px));
-    qx = mad_w(v.z, y.y, mad_w(v.w, y.x, qx));
+    rx = mad_w(v.y, y.x, rx);
+    ry = mad_w(v.w, y.z, ry);
+    px = mad_w(v.y, y.z, px);
+    qx = mad_w(v.w, y.x, qx);
+    rh = mad_w(v.z, y.z, rh);
+    rx = mad_w(v.x, y.y, rx);
+    ry = mad_w(v.z, y.w, ry);
+    px = mad_w(v.x, y.w, px);
+    qx = mad_w(v.z, y.y, qx);
   }
   // |hh| <= 2^58 over a lane's CG_U points: the sum over 16 lanes fits
-  __device__ __forceinline__ long long re() const { return fx_sum(rh, rx); }
+  __device__ __forceinline__ long long re() const { return fx_sum(rh, rx + ry); }
   __device__ __forceinline__ long long im() const { return fx_sum(ph - qh, px - qx); }
 };
 // limb sums of c v
@@ -805,7 +812,7 @@ hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, in
   // One kernel while a tile's rows fit the shared memory of half an SM, with as
   // many blocks per SM as hold them: what it lacks is warps, not room for the
   // next tile's rows (2^24 points, j = 22: four blocks of 24 rows 1703 us, three
-  // of 34 1727, two of 52 2001, two kernels 2270; j = 39: 3290 against 3780).
+  // of 34 1727, two of 52 2001, two kernels 2270; j = 39: 3050 against 3780).
   if (j + 1 > CG_FUSED) {
     HZ_TRY(launch_cgs<CG_UPDATE>(Q, cgs_blocks(Q.ntiles, nrhs, 4), CG_ROWS, w, wstride, j, nrhs,
                                  S1, ldS, sigma, ldsig, active, partial, nullptr, nullptr, st));
