@@ -161,9 +161,9 @@ static hz_status ensure_planes(hz_plan* p, int prec) {
 // Shape of the complex64 symbol pass for a last axis of N points and `points`
 // points over all right-hand sides, as (nodes per block, columns per thread).
 // Blocks of four nodes read the spectrum once for four planes and pay where
-// there are enough blocks without them (256^3 1393 -> 1257 us, 512^2 x 16
-// right-hand sides 266 -> 247, 2048^2 559 -> 509, 64^3 x 8 162 -> 149; but
-// 1024^2 104 -> 113, 128^3 163 -> 169).  A pair of columns needs the registers
+// there are enough blocks without them (512^2 x 16 right-hand sides 266 -> 247 us, 2048^2 559 -> 509, 64^3 x 8 162 -> 149; but
+// 1024^2 104 -> 113); columns of 128 and 256 loop over more nodes with the
+// spectrum in shared memory (256^3 1390 -> 1178, 128^3 x 4 572 -> 554).  A pair of columns needs the registers
 // of two lines: threads with 24 or 30 elements (factors 3 and 5) do better
 // with one column on small grids (192^2 20.8 -> 17.6 us, 360 x 480 41 -> 34,
 // 720^2 122 -> 111) and with half blocks or four nodes on large ones
@@ -181,6 +181,8 @@ static void sym_shape(int N, long points, int* kpb, int* pair) {
     }
   } else if (N == 96 || N == 192) {
     *pair = points < (1l << 17) ? 0 : 2;
+  } else if (N <= 256 && N >= 128 && points >= (1l << 22)) {
+    *kpb = N == 256 ? 16 : 8;  // line_sym_inv_loop_kernel
   } else if (points >= (1l << 21)) {
     if (N == 256 || N == 512 || N == 2048) *kpb = 4;
     if (N == 64) {

@@ -275,6 +275,26 @@ hz_status line_sym_inv_t(const void* vhat, void* planes, int nx, long outer, lon
                          int kpb, int pair) {
   using C = LineCfg<R, N>;
   using V = typename cvec<R>::T;
+  if constexpr (std::is_same<R, float>::value && (N == 128 || N == 256)) {
+    // more nodes than that: the loop over nodes with the spectrum in shared memory
+    if (kpb > SYM_KPB_MAX && tw2 && nx % 2 == 0) {
+      constexpr int TB = C::template tb_p<1>();
+      constexpr int NT = TB * C::template tpl_p<1>();
+      auto k = symD ? line_sym_inv_loop_kernel<N, TB, true> : line_sym_inv_loop_kernel<N, TB, false>;
+      constexpr size_t smem = C::col_pair_smem(TB) + size_t(N) * TB * 16 + size_t(N) * 12;
+      HZ_TRY(smem_attr(k, smem));
+      const int ntile = (nx / 2 + TB - 1) / TB;
+      HZ_CUDA(launch_pdl(k, dim3(unsigned(ntile * outer), unsigned((K + kpb - 1) / kpb), unsigned(batch)),
+                         dim3(NT), smem, st, static_cast<const float2*>(vhat),
+                         static_cast<float2*>(planes), nx, ntile, S, ostride, n, K, kpb,
+                         static_cast<const float*>(xi2_x), static_cast<const float*>(xi2_o),
+                         static_cast<const float*>(xi2_l), static_cast<const float2*>(symA),
+                         static_cast<const float2*>(symG), static_cast<const float*>(symD), smask,
+                         smO, smS, static_cast<const float4*>(tw2), active));
+      HZ_CUDA(cudaGetLastError());
+      return HZ_OK;
+    }
+  }
   // nodes per block: 1, 2 or 4
   kpb = kpb >= 4 ? 4 : (kpb >= 2 ? 2 : 1);
   if constexpr (std::is_same<R, float>::value) {

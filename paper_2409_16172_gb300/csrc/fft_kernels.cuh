@@ -118,16 +118,6 @@ __device__ __forceinline__ float recip(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// FP64: the MUFU approximation refined by three Newton-Raphson steps for
-// 1/x, r <- r + r (1 - x r), each of which doubles the number of correct bits.
-__device__ __forceinline__ double recip(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-#pragma unroll
-  for (int it = 0; it < 3; ++it) r = fma(r, fma(-x, r, 1.0), r);
-  return r;
-}
-
 template <typename R> struct RecT;
 template <> struct RecT<float> { using T = uint32_t; };
 template <> struct RecT<double> { using T = double; };
@@ -661,6 +651,31 @@ line_sym_inv_kernel(const typename cvec<R>::T* __restrict__ vhat,
 }
 
 
+// vhat q_k = vhat conj(den) / |den|^2,  den = A - G |xi|^2, of two columns
+template <bool HERM>
+__device__ __forceinline__ PV pair_symbol(const PV& sp, f2 s2, f2 AX, f2 AY, f2 NGX, f2 NGY, float D) {
+  PV den;
+  den.x = fma2(NGX, s2, AX);
+  den.y = fma2(NGY, s2, AY);
+  const f2 nrm = fma2(den.x, den.x, den.y * den.y);
+  const f2 inv = f2_make(recip(f2_lo(nrm)), recip(f2_hi(nrm)));
+  const PV q = cmulc(sp, den);
+  PV r;
+  r.x = q.x * inv;
+  r.y = q.y * inv;
+  if (HERM && D != 0.0f) {
+    // derivative plane of the Hermite basis: vhat dq/dc = vhat q (D |xi|^2 q)
+    PV qv;
+    qv.x = den.x * inv;
+    qv.y = neg2(den.y) * inv;
+    r = cmul(r, qv);
+    const f2 ds = f2_splat(D) * s2;
+    r.x = r.x * ds;
+    r.y = r.y * ds;
+  }
+  return r;
+}
+
 // The complex64 symbol pass with two adjacent columns per thread (x, x + 1;
 // nx even), their values paired in f32x2 registers (PV): the same arithmetic
 // per column as line_sym_inv_kernel, in packed FP32 instructions, 16-byte
@@ -741,28 +756,8 @@ line_sym_inv_pair_kernel(const float2* __restrict__ vhat, float2* __restrict__ p
       mb[(e * KPB) / 32] |= bits << ((e * KPB) % 32);
     }
   }
-  // vhat q_k = vhat conj(den) / |den|^2,  den = A - G |xi|^2
   auto symbol = [](const PV& sp, f2 s2, f2 AX, f2 AY, f2 NGX, f2 NGY, float D) {
-    PV den;
-    den.x = fma2(NGX, s2, AX);
-    den.y = fma2(NGY, s2, AY);
-    const f2 nrm = fma2(den.x, den.x, den.y * den.y);
-    const f2 inv = f2_make(recip(f2_lo(nrm)), recip(f2_hi(nrm)));
-    const PV q = cmulc(sp, den);
-    PV r;
-    r.x = q.x * inv;
-    r.y = q.y * inv;
-    if (HERM && D != 0.0f) {
-      // derivative plane of the Hermite basis: vhat dq/dc = vhat q (D |xi|^2 q)
-      PV qv;
-      qv.x = den.x * inv;
-      qv.y = neg2(den.y) * inv;
-      r = cmul(r, qv);
-      const f2 ds = f2_splat(D) * s2;
-      r.x = r.x * ds;
-      r.y = r.y * ds;
-    }
-    return r;
+    return pair_symbol<HERM>(sp, s2, AX, AY, NGX, NGY, D);
   };
   auto store = [&](int k, int kk, PV (&v)[E]) {
     if (!valid) return;
@@ -815,6 +810,84 @@ line_sym_inv_pair_kernel(const float2* __restrict__ vhat, float2* __restrict__ p
       for (int e = 0; e < E; ++e) v[e] = symbol(spec[e], s2[e], AX, AY, NGX, NGY, D);
       F::run_regs(sm + col, t, v, tw2);
       store(k, k - k0, v);
+    }
+  }
+}
+
+// The paired symbol pass with a block's part of the spectrum in shared memory
+// (each thread's own elements, so without a barrier) and a loop over kpb
+// nodes: the same arithmetic as line_sym_inv_pair_kernel.  One-node blocks
+// wait on the spectrum's loads from L2 (long scoreboard 4.1 of 9.3 cycles per
+// issue at 256^3); blocks that keep it in registers over four nodes have half
+// the warps.  Whole apply at 256^3, K = 16: one node per block 1390 us, four
+// in registers 1250, this 1178; 128^3 x 4 right-hand sides 572, 583, 554;
+// 512-point columns no better than four in registers.
+template <int N, int TB, bool HERM>
+__global__ void __launch_bounds__(TB * LineCfg<float, N>::template tpl_p<1>(), 3)
+line_sym_inv_loop_kernel(const float2* __restrict__ vhat, float2* __restrict__ planes, int nx,
+                         int ntile, long S, long ostride, long n, int K, int kpb,
+                         const float* __restrict__ xi2_x, const float* __restrict__ xi2_o,
+                         const float* __restrict__ xi2_l, const float2* __restrict__ symA,
+                         const float2* __restrict__ symG, const float* __restrict__ symD,
+                         const unsigned long long* __restrict__ smask, long smO, long smS,
+                         const float4* __restrict__ tw2, const int* __restrict__ active) {
+  pdl_wait();
+  using F = LineFFT<float, N, +1, TB, false, typename LineCfg<float, N>::template PPK<1>, PV>;
+  constexpr int E = F::E, NT = TB * F::TPL;
+  if (active && !active[blockIdx.z]) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  PV* sm = reinterpret_cast<PV*>(smem_raw);
+  float4* spec = reinterpret_cast<float4*>(smem_raw + LineCfg<float, N>::col_pair_smem(TB));
+  unsigned long long* msk = reinterpret_cast<unsigned long long*>(spec + E * NT);
+  float* xl = reinterpret_cast<float*>(msk + N);
+  const int col = threadIdx.x % TB, t = threadIdx.x / TB;
+  const int tile = blockIdx.x % ntile;
+  const long o = blockIdx.x / ntile;
+  const int k0 = blockIdx.y * kpb, k1 = min(K, k0 + kpb);
+  const long rhs = blockIdx.z;
+  const int x = 2 * (tile * TB + col);
+  const bool valid = x < nx;
+  const long off = o * ostride + x;
+  const float2* src = vhat + rhs * n + off;
+  const int Sl = int(S);
+  const float so = xi2_o ? xi2_o[o] : 0.0f;
+  const float sx0 = (valid ? xi2_x[x] : 0.0f) + so, sx1 = (valid ? xi2_x[x + 1] : 0.0f) + so;
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    cp_async16(spec + e * NT + threadIdx.x,
+               valid ? src + F::stage0_index(t, e) * Sl : src - x);
+  cp_async_commit();
+  for (int i = threadIdx.x; i < N; i += NT) {
+    msk[i] = smask[o * smO + i * int(smS)];
+    xl[i] = xi2_l[i];
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
+#pragma unroll 1
+  for (int k = k0; k < k1; ++k) {
+    const float2 A = symA[k], G = symG[k];
+    const float D = HERM ? symD[k] : 0.0f;
+    const f2 AX = f2_splat(A.x), AY = f2_splat(A.y), NGX = f2_splat(-G.x), NGY = f2_splat(-G.y);
+    PV v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const float4 a = spec[e * NT + threadIdx.x];
+      PV sp;
+      sp.x = f2_make(a.x, a.z);
+      sp.y = f2_make(a.y, a.w);
+      const float l = xl[F::stage0_index(t, e)];
+      v[e] = pair_symbol<HERM>(sp, f2_make(sx0 + l, sx1 + l), AX, AY, NGX, NGY, D);
+    }
+    F::run_regs(sm + col, t, v, tw2);
+    if (valid) {
+      float2* dst = planes + (rhs * K + k) * n + off;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int p = F::out_index(t, e);
+        if ((msk[p] >> k) & 1ull)
+          *reinterpret_cast<float4*>(dst + p * Sl) =
+              make_float4(f2_lo(v[e].x), f2_lo(v[e].y), f2_hi(v[e].x), f2_hi(v[e].y));
+      }
     }
   }
 }
