@@ -816,6 +816,7 @@ hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, in
   if (j + 1 > CG_FUSED) {
     HZ_TRY(launch_cgs<CG_UPDATE>(Q, cgs_blocks(Q.ntiles, nrhs, 4), CG_ROWS, w, wstride, j, nrhs,
                                  S1, ldS, sigma, ldsig, active, partial, nullptr, nullptr, st));
+    count_launches(1);  // the phase counts two
     return launch_dots(Q, w, wstride, j, nrhs, active, partial, S2, ldS, st);
   }
   const int per_sm = j + 1 <= CG_ROWS ? 4 : (j + 1 <= 34 ? 3 : 2);
