@@ -497,20 +497,16 @@ __device__ __forceinline__ double2 cmul_d(double2 a, double2 b) {
 __device__ __forceinline__ double2 cfma_d(double2 a, double2 b, double2 c) {  // a b + c
   return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
 }
-// 1/sqrt(x) for x > 0: the MUFU approximation refined by three Newton-Raphson
-// steps y <- y + y (1 - x y^2) / 2 (each doubles the correct bits).  The
-// Givens kernel runs in one warp, where every FP64 instruction holds the
-// sub-partition's FP64 unit for ~64 cycles; this takes fewer of them than a
-// square root followed by a division.
+// 1/sqrt(x) for x > 0: the MUFU approximation (about 20 bits) and one step of
+// third order, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - x y^2.  Every FP64
+// instruction of a warp holds the sub-partition's FP64 unit for ~64 cycles;
+// this takes fewer of them than a square root followed by a division, or than
+// second-order steps.
 __device__ __forceinline__ double rsqrt_nr(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-#pragma unroll
-  for (int it = 0; it < 3; ++it) {
-    const double e = fma(-x * y, y, 1.0);
-    y = fma(0.5 * y, e, y);
-  }
-  return y;
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y, e * fma(0.375, e, 0.5), y);
 }
 // max(|a|, |b|) of finite doubles as an integer max of the magnitude bits
 // (IEEE order of non-negative doubles is that of their bit patterns), off the
@@ -532,21 +528,35 @@ constexpr int GT = 128;
 //   x_0 = h_0,  x_{i+1} = -conj(s_i) x_i + c_i h_{i+1},  r_i = c_i x_i + s_i h_{i+1},
 // evaluated by the first warp as a scan of affine maps (each lane composes a contiguous
 // chunk, a shuffle scan composes the chunks) instead of j serial steps.
-// First |w|^2 from the update's nblk block sums (fixed order), by all warps.
+// The other warps meanwhile sum |w|^2 from the update's nblk block sums (fixed
+// order) and take its root, and divide the history's entry: one warp doing it
+// all in turn held its FP64 unit for 2.3 us a step longer (128^2, 29 steps:
+// solve 1759 -> 1690 us).
 __global__ void __launch_bounds__(GT)
 givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
   pdl_wait();
   const int b = blockIdx.x;
   if (!ks.active[b]) return;
-  __shared__ double nsum[GT / 32 + 1];
-  {
-    double v[1] = {0.0};
-    for (int i = threadIdx.x; i < nblk; i += GT) v[0] += partial[long(b) * nblk + i];
-    block_sum<1, GT>(v, nsum);
+  __shared__ double wsum[GT / 32], shn[3];  // warp sums; |w|^2, 1 / |w|, estimate
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp > 0) {
+    double v = 0.0;
+    for (int i = threadIdx.x - 32; i < nblk; i += GT - 32) v += partial[long(b) * nblk + i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) wsum[warp] = v;
+    asm volatile("bar.sync 1, %0;" ::"n"(GT - 32) : "memory");
+    if (threadIdx.x == 32) {
+      double q = wsum[1];
+      for (int i = 2; i < GT / 32; ++i) q += wsum[i];
+      shn[0] = q;  // |w|^2 after orthogonalisation
+      shn[1] = q > 0.0 ? rsqrt_nr(q) : 0.0;
+    }
+    __syncthreads();
+    __syncthreads();
+    if (threadIdx.x == 32) ks.hist[long(b) * ks.m + j] = shn[2] / ks.bnorm[b];
+    return;
   }
-  const double hn2 = nsum[GT / 32];  // |w|^2 after orthogonalisation
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
   const int m = ks.m;
   __shared__ double2 col[HZ_MAX_RESTART + 2];   // h, the new column before rotation
   __shared__ double2 rcol[HZ_MAX_RESTART + 2];  // rotated column
@@ -569,7 +579,6 @@ givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) hbits = max(hbits, __shfl_xor_sync(0xffffffffu, hbits, o));
   const double hmax = __longlong_as_double(hbits);
-  bad = __any_sync(0xffffffffu, bad) || !isfinite(hn2);
   __syncwarp();
   // chunk of maps i in [i0, i1) of this lane; composite F(x) = A x + B
   const int per = (j + 31) / 32;
@@ -579,12 +588,17 @@ givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
     const double2 al = make_double2(-sn[i].x, sn[i].y);  // -conj(s_i)
     const double c = cs[i];
     const double2 be = make_double2(c * col[i + 1].x, c * col[i + 1].y);
-    A = cmul_d(al, A);
-    B = cfma_d(al, B, be);
+    if (i == i0) {
+      A = al;
+      B = be;
+    } else {
+      A = cmul_d(al, A);
+      B = cfma_d(al, B, be);
+    }
   }
-  // inclusive scan over lanes: G_l = F_l o F_{l-1} o ... o F_0
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
+  // inclusive scan over the lanes that hold a chunk: G_l = F_l o ... o F_0
+  const int last = per ? (j - 1) / per : 0;
+  for (int o = 1; o <= last; o <<= 1) {
     const double2 Ap = shfl_up_d2(A, o), Bp = shfl_up_d2(B, o);
     if (lane >= o) {
       B = cfma_d(A, Bp, B);
@@ -604,12 +618,15 @@ givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
     rcol[i] = cfma_d(sv, h1, make_double2(c * x.x, c * x.y));
     x = cfma_d(make_double2(-sv.x, sv.y), x, make_double2(c * h1.x, c * h1.y));
   }
-  const double2 xall = cfma_d(A, h0, B);  // lane 31 holds the full composition
-  const double2 a = make_double2(__shfl_sync(0xffffffffu, xall.x, 31), __shfl_sync(0xffffffffu, xall.y, 31));
-  __syncwarp();
+  const double2 xall = cfma_d(A, h0, B);  // lane last holds the full composition
+  const double2 a =
+      make_double2(__shfl_sync(0xffffffffu, xall.x, last), __shfl_sync(0xffffffffu, xall.y, last));
+  __syncthreads();  // |w|
+  const double hn2 = shn[0];
+  bad = __any_sync(0xffffffffu, bad) || !isfinite(hn2);
   if (lane == 0) {
     // h_{j+1,j} = hn = |w|; sigma_{j+1} = 1 / hn normalises the next vector
-    const double inv_hn = hn2 > 0.0 ? rsqrt_nr(hn2) : 0.0;
+    const double inv_hn = shn[1];
     const double hn = hn2 * inv_hn;
     ks.Hraw[(long(b) * m + j) * (m + 1) + j + 1] = make_double2(hn, 0.0);
     const bool happy = hn <= 1e-14 * hmax;
@@ -644,7 +661,7 @@ givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
     const double gn2 = fma(gn.x, gn.x, gn.y * gn.y);
     const double est = gn2 > 0.0 ? gn2 * rsqrt_nr(gn2) : 0.0;
     ks.est[b] = est;
-    ks.hist[long(b) * m + j] = est / ks.bnorm[b];
+    shn[2] = est;
     ks.jend[b] = j + 1;
     bad |= !isfinite(est) || !isfinite(r.x) || !isfinite(r.y);
     int act = 1;
@@ -659,7 +676,7 @@ givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
       atomicSub(ks.n_active, 1);
     }
   }
-  __syncwarp();
+  __syncthreads();  // the estimate
   for (int i = lane; i <= j + 1; i += 32) colg[i] = rcol[i];
 }
 
