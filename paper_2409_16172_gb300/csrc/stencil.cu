@@ -122,6 +122,7 @@ stencil_kernel(const InT* __restrict__ x, double2* __restrict__ y, const double2
 // ---------------------------------------------------------------------------
 constexpr int SW = 8;          // warps per block
 constexpr int FS_TOP = 56;
+constexpr int FS_KEEP = 3;     // bits of the result kept below 2^62 units
 
 template <bool D3> struct FsTile {
   static constexpr int TY = D3 ? 8 : 32, TZ = D3 ? 8 : 1;
@@ -312,12 +313,14 @@ stencil_fx_kernel(const InT* __restrict__ x, double2* __restrict__ y, const doub
         const int nz_ = -G.z, nw = -G.w;
         const long long rh = mad_w(k.w2h, vxh, mad_w(nz_, bh, mul_w(G.x, ah)));
         const long long ih = mad_w(k.w2h, vyh, mad_w(G.z, ah, mul_w(G.x, bh)));
-        long long rm = (mad_w(nw, bl, mul_w(G.y, al)) >> 31) + (mul_w(k.w2l, vxl) >> 31);
-        long long im = (mad_w(G.w, al, mul_w(G.y, bl)) >> 31) + (mul_w(k.w2l, vyl) >> 31);
+        // rounded at the last bit kept: |g L + omega^2 v| < 2^121.2, 62.2 bits left
+        constexpr long long half = 1ll << (30 - FS_KEEP);
+        long long rm = (mad_w(nw, bl, mul_w(G.y, al)) >> 31) + (mad_w(k.w2l, vxl, half << 31) >> 31);
+        long long im = (mad_w(G.w, al, mul_w(G.y, bl)) >> 31) + (mad_w(k.w2l, vyl, half << 31) >> 31);
         rm = mad_w(G.x, al, mad_w(G.y, ah, mad_w(nz_, bl, mad_w(nw, bh, mad_w(k.w2h, vxl, mad_w(k.w2l, vxh, rm))))));
         im = mad_w(G.x, bl, mad_w(G.y, bh, mad_w(G.z, al, mad_w(G.w, ah, mad_w(k.w2h, vyl, mad_w(k.w2l, vyh, im))))));
-        yr = fx_to((rh << 2) + (rm >> 29), ke);
-        yi = fx_to((ih << 2) + (im >> 29), ke);
+        yr = fx_to((rh << FS_KEEP) + (rm >> (31 - FS_KEEP)), ke);
+        yi = fx_to((ih << FS_KEEP) + (im >> (31 - FS_KEEP)), ke);
       } else {
         auto d = [&](int i) {
           return make_double2(__longlong_as_double(c[i].x), __longlong_as_double(c[i].y));
@@ -410,8 +413,8 @@ bool fx_consts(const StencilConsts& c, int dim, int uq, FxStencil* k) {
       limbs31(std::llrint(std::ldexp(kap[i], -weight_unit(c))), &k->kh[i], &k->kl[i]);
   }
   k->qg = std::ldexp(1.0, uq);
-  // a 31 x 31 bit product's high part counts 2^62 units; the sums keep two more bits
-  k->k_out = 62 - 2 + uq + ul - FS_TOP - 1023;
+  // a 31 x 31 bit product's high part counts 2^62 units; the sums keep FS_KEEP more bits
+  k->k_out = 62 - FS_KEEP + uq + ul - FS_TOP - 1023;
   return true;
 }
 
