@@ -118,7 +118,7 @@ stencil_kernel(const InT* __restrict__ x, double2* __restrict__ y, const double2
 // the FP64 formula.  It is bound by the integer multiply-add pipe, which also
 // takes the 64-bit additions (62 lanes per clock and SM, about 130 a point in
 // 2D).  2400^2 damped, c128 input: 180 -> 82 us (3.9 TB/s); 192^3, c64 input:
-// 277 -> 113 us (2.5 TB/s).
+// 277 -> 115 us (2.5 TB/s).
 // ---------------------------------------------------------------------------
 constexpr int SW = 8;          // warps per block
 constexpr int FS_TOP = 56;
