@@ -12,8 +12,13 @@
 // so the stage cannot overflow 2^61; after it the largest component of the
 // block is known (one reduction that rides on the stage's barrier) and the
 // next stage's reads shift all values to the top of its range again.  A value
-// thus keeps at least 55 bits below the largest of its block in every stage,
-// and the error of a transform stays below that of FP64 stages.
+// thus keeps at least 55 bits below the largest of its block in every stage.
+// Values, products and shifts are rounded to nearest: a truncation's bias adds
+// up over a line, above all where a spectrum is a few large entries.  Whole
+// apply against extended precision, here (cut instead of rounded; FP64 stages):
+// 40 x 48 x 60 noise 3.6e-16 (5.2; 4.7), wide bump 2.6 (5.1; 2.8), plane wave 2.3
+// (3.3; 2.4); 240 x 360 noise 3.8 (4.3; 5.7), plane wave 2.8 (5.1; 3.8).
+// Rounding costs no time (480 x 720, K = 8: 193 -> 190 us).
 // A block's lines belong to one right-hand side: its results do not depend on
 // what else is in the batch.
 //
@@ -42,27 +47,33 @@ template <int M, typename F> __device__ __forceinline__ void static_for(F&& f) {
 }
 
 // ---- products with numbers of modulus <= 1, held times 2^61 -----------------
-__device__ __forceinline__ int l31h(long long v) { return int(v >> 31); }
-__device__ __forceinline__ int l31l(long long v) { return int(unsigned(v) & 0x7fffffffu); }
+// Limbs v = h 2^31 + l, l symmetric about zero (as those of the twiddle table
+// and of the constants): the partial products l l are then left out without
+// a bias.
+__device__ __forceinline__ int l31l(long long v) { return int(unsigned(v) << 1) >> 1; }
+__device__ __forceinline__ int l31h(long long v) { return int(v >> 31) - (l31l(v) >> 31); }
+constexpr int q31h(long long c) { return int((c + (1ll << 30)) >> 31); }
+constexpr int q31l(long long c) { return int(c - q31h(c) * (1ll << 31)); }
 // constants times 2^61, rounded
 constexpr long long q61(double c) {
   return c < 0 ? -q61(-c) : (long long)(c * 2305843009213693952.0 + 0.5);
 }
-// (hh 2^62 + m 2^31) / 2^61; the lowest partial products (two units) are left out
+// (hh 2^62 + m 2^31) / 2^61 to the nearest integer, where m was begun with
+// half; the lowest partial products (below one unit, of mean zero) are left out
+constexpr long long HALF61 = 1ll << 29;
 __device__ __forceinline__ long long join61(long long hh, long long m) { return (hh << 1) + (m >> 30); }
 
 template <long long C> __device__ __forceinline__ long long mulq(long long v) {
-  constexpr int ch = int(C >> 31), cl = int(C & 0x7fffffff);
+  constexpr int ch = q31h(C), cl = q31l(C);
   const int h = l31h(v), l = l31l(v);
-  return join61(mad_w(h, ch, 0), mad_w(h, cl, mad_w(l, ch, 0)));
+  return join61(mad_w(h, ch, 0), mad_w(h, cl, mad_w(l, ch, HALF61)));
 }
 // C1 v + C2 w
 template <long long C1, long long C2> __device__ __forceinline__ long long mulq2(long long v, long long w) {
-  constexpr int ah = int(C1 >> 31), al = int(C1 & 0x7fffffff);
-  constexpr int bh = int(C2 >> 31), bl = int(C2 & 0x7fffffff);
+  constexpr int ah = q31h(C1), al = q31l(C1), bh = q31h(C2), bl = q31l(C2);
   const int h = l31h(v), l = l31l(v), p = l31h(w), q = l31l(w);
   return join61(mad_w(p, bh, mad_w(h, ah, 0)),
-                mad_w(p, bl, mad_w(q, bh, mad_w(h, al, mad_w(l, ah, 0)))));
+                mad_w(p, bl, mad_w(q, bh, mad_w(h, al, mad_w(l, ah, HALF61)))));
 }
 template <long long C, long long D> __device__ __forceinline__ CI cmulq(CI a) {  // a (C + i D)
   return CI{mulq2<C, -D>(a.x, a.y), mulq2<D, C>(a.x, a.y)};
@@ -74,9 +85,9 @@ template <int S> __device__ __forceinline__ CI twiddle_int(CI a, int4 w) {
   const int nh = S > 0 ? w.z : -w.z, nl = S > 0 ? w.w : -w.w;  // and its negative
   CI r;
   r.x = join61(mad_w(yh, nh, mad_w(xh, w.x, 0)),
-               mad_w(yh, nl, mad_w(yl, nh, mad_w(xh, w.y, mad_w(xl, w.x, 0)))));
+               mad_w(yh, nl, mad_w(yl, nh, mad_w(xh, w.y, mad_w(xl, w.x, HALF61)))));
   r.y = join61(mad_w(yh, w.x, mad_w(xh, ih, 0)),
-               mad_w(yh, w.y, mad_w(yl, w.x, mad_w(xh, il, mad_w(xl, ih, 0)))));
+               mad_w(yh, w.y, mad_w(yl, w.x, mad_w(xh, il, mad_w(xl, ih, HALF61)))));
   return r;
 }
 
@@ -238,16 +249,16 @@ HZ_IPLAN(4800, 10, 10, 8, 6)
 #undef HZ_IPLAN
 
 // ---- doubles to and from a block's integers -----------------------------------
-// x 2^(top + 1023 - E), truncated; E >= exponent of x, 52 <= top <= 62
+// x 2^(top + 1023 - E) to the nearest integer; E >= exponent of x, 52 <= top <= 61
 __device__ __forceinline__ long long int_of(double x, int E, int top) {
   const int hi = __double2hiint(x);
   const unsigned lo = unsigned(__double2loint(x));
   const int ex = (hi >> 20) & 0x7ff;
   const unsigned mh = ex == 0 ? 0u : unsigned((hi & 0xfffff) | 0x100000);
-  unsigned long long t = (static_cast<unsigned long long>(mh) << 32 | (ex == 0 ? 0u : lo)) << (top - 52);
+  unsigned long long t = (static_cast<unsigned long long>(mh) << 32 | (ex == 0 ? 0u : lo)) << (top - 51);
   asm("shr.u64 %0, %0, %1;" : "+l"(t) : "r"(E - ex));
   const long long s = hi >> 31;
-  return (static_cast<long long>(t) ^ s) - s;
+  return (static_cast<long long>((t + 1) >> 1) ^ s) - s;
 }
 // t 2^k: zero below the normal range, infinity above it
 __device__ __forceinline__ double double_of(long long t, int k) {
@@ -313,8 +324,9 @@ __device__ __forceinline__ void int_stage(CI* src, CI* dst, int* red, int E0, in
 #pragma unroll
         for (int r = 0; r < RAD; ++r) x[r] = CI{x[r].x << sh, x[r].y << sh};
       } else {
+        const long long half = 1ll << (-sh - 1);
 #pragma unroll
-        for (int r = 0; r < RAD; ++r) x[r] = CI{x[r].x >> -sh, x[r].y >> -sh};
+        for (int r = 0; r < RAD; ++r) x[r] = CI{(x[r].x + half) >> -sh, (x[r].y + half) >> -sh};
       }
     }
     const int k = NS > 1 ? j % NS : 0;

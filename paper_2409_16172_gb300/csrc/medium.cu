@@ -631,11 +631,11 @@ extern "C" hz_status hz_create_medium(const hz_grid* grid, const double* c, cons
     std::vector<double> xi;
     twiddles(N, tw);
     xi2_table(N, m->L, interp->symbol_kind, xi);
-    std::vector<int4> twi(N);  // times 2^61, in limbs of 31 bits (fft_int.cuh)
+    std::vector<int4> twi(N);  // times 2^61, in limbs of 31 bits, the low one symmetric (fft_int.cuh)
     auto limbs = [](double v, int* hi, int* lo) {
       const long long q = std::llrint(std::ldexp(v, 61));
-      *hi = int(q >> 31);
-      *lo = int(q & 0x7fffffff);
+      *hi = int((q + (1ll << 30)) >> 31);
+      *lo = int(q - *hi * (1ll << 31));
     };
     std::vector<float2> twf(N);
     std::vector<float4> twp(N);
