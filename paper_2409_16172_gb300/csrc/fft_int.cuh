@@ -19,8 +19,8 @@
 // 40 x 48 x 60 noise 3.6e-16 (5.2; 4.7), wide bump 2.6 (5.1; 2.8), plane wave 2.3
 // (3.3; 2.4); 240 x 360 noise 3.8 (4.3; 5.7), plane wave 2.8 (5.1; 3.8).
 // Rounding costs no time (480 x 720, K = 8: 193 -> 190 us).
-// A block's lines belong to one right-hand side: its results do not depend on
-// what else is in the batch.
+// A block's lines belong to one right-hand side, and which lines share a block
+// does not depend on the call's other right-hand sides: neither do results.
 //
 // Stages ping-pong between two shared-memory copies of the lines; a work item
 // is one butterfly, so a thread holds one radix of elements, and any thread
