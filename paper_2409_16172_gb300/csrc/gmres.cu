@@ -122,7 +122,8 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
   const int prec = p->opts.precision;
   const double tol = p->opts.tol;
   const long ldb = B;  // basis vector i of rhs b at slot i * B + b
-  const Basis Q{reinterpret_cast<int4*>(p->V), p->ev, ldb, n, (n + HZ_FX_TILE - 1) / HZ_FX_TILE};
+  const Basis Q{reinterpret_cast<int4*>(p->V), p->ev, ldb, n, (n + HZ_FX_TILE - 1) / HZ_FX_TILE,
+                p->opts.no_precond == 0};
   double2* W = p->V + long(m) * ldb * n;  // the current vector in FP64 (slot m)
 
   HZ_TRY(check_device(med));

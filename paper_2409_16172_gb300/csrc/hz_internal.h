@@ -283,8 +283,8 @@ struct hz_plan {
   int planes_prec = 1;     // precision the planes buffer is sized for (0 = c128)
   // Krylov workspace (FP64)
   double2* V = nullptr;    // [(m+1)][max_nrhs][n]: slots 0 .. m-1 the unnormalised basis
-                           // vectors in block fixed-point form (16 bytes a point), slot m
-                           // the current vector in FP64
+                           // vectors, 16 bytes a point (kernels.h's Basis), slot m the
+                           // current vector in FP64
   int* ev = nullptr;       // [m][max_nrhs][tiles] exponents of the basis tiles
   void* Z = nullptr;       // [m][max_nrhs][n] preconditioned vectors (c64 or unused)
   double2* u = nullptr;    // staged solution for host buffers [max_nrhs][n]

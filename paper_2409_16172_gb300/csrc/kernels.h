@@ -91,13 +91,14 @@ hz_status launch_residual(const hz_medium* m, const double2* u, const double2* f
                           cudaStream_t st);
 
 int krylov_blocks(long n, int nrhs, int nchunk);
-// Arnoldi basis in block fixed-point form (fixed.cuh): vector i of
-// right-hand side b at V + (i ldb + b) n, its tile exponents at
-// ev + (i ldb + b) ntiles.
+// Arnoldi basis: vector i of right-hand side b at V + (i ldb + b) n.  fixed:
+// in block fixed-point form (fixed.cuh), with tile exponents at
+// ev + (i ldb + b) ntiles; else in FP64.
 struct Basis {
   int4* V;
   int* ev;
   long ldb, n, ntiles;
+  bool fixed;
 };
 // S = raw sums of conj(V_i) w, i <= j (pass 1)
 hz_status launch_dots(const Basis& Q, double2* w, long wstride, int j, int nrhs, const int* active,

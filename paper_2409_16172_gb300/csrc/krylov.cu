@@ -8,9 +8,17 @@
 //   h_i   = <v_i, w> = sigma_i * sum conj(V_i) w          (dots)
 //   w    -= sum_i h_i v_i = sum_i (sigma_i h_i) V_i         (update)
 // so no pass ever rescales a stored vector.
-// Layout: V[(i * ldb + b) * n + p] for basis vector i, right-hand side b, in
-// the block fixed-point form of fixed.cuh (16 bytes a point); the current
-// vector w is FP64.
+// Layout: V[(i * ldb + b) * n + p] for basis vector i, right-hand side b, 16
+// bytes a point; the current vector w is FP64.  Two forms of the basis:
+//   block fixed point (fixed.cuh), where the preconditioner's transforms make
+//     the vectors: a transform's rounding errors are of one size all over the
+//     grid, so that a unit of 2^-54 of the largest of 128 neighbours costs
+//     nothing (complex128 solves of 16 steps: solution and Hessenberg entries
+//     as close to extended precision as in FP64)
+//   FP64, for the unpreconditioned method: its vectors come from the operator
+//     alone, which keeps the bits of values however small they are beside
+//     their neighbours (a point source's field 1e-8 of its largest value:
+//     relative error 2e-15 in FP64, 2e-6 in block fixed point; 128^2, 40 steps)
 #include <math.h>
 
 #include <algorithm>
@@ -443,7 +451,167 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same on an FP64 basis, bound by the FP64 pipe (2^24 points: 2.1-2.5 TB/s
+// of basis).
+// ---------------------------------------------------------------------------
+constexpr int VC = 8;  // basis vectors per dots block at most
+
+// Sums of conj(V_i) w for i in [i0, i0 + nv), i0 = blockIdx.z vpc, nv =
+// min(vpc, j + 1 - i0), vpc <= VC.  grid (blocks, rhs, chunks).  The next
+// point's operands are loaded before the current point's FMAs, so that the
+// FP64 pipe does not wait on memory.
+__global__ void __launch_bounds__(KT, 2)
+dots_kernel(const double2* __restrict__ V, long ldb, const double2* __restrict__ w, long wstride,
+            long n, int j, int vpc, const int* __restrict__ active, double2* __restrict__ partial) {
+  pdl_wait();
+  const int b = blockIdx.y;
+  if (!active[b]) return;
+  const int i0 = blockIdx.z * vpc;
+  const int nv = min(vpc, j + 1 - i0);
+  double sum[2 * VC];
+#pragma unroll
+  for (int c = 0; c < 2 * VC; ++c) sum[c] = 0.0;
+  const double2* wb = w + b * wstride;
+  const double2* Vb = V + (long(i0) * ldb + b) * n;
+  const long vs = ldb * n;
+  const long step = long(gridDim.x) * KT;
+  long p = long(blockIdx.x) * KT + threadIdx.x;
+  double2 x, v[VC];
+  if (p < n) {
+    x = wb[p];
+#pragma unroll
+    for (int c = 0; c < VC; ++c)
+      if (c < nv) v[c] = Vb[c * vs + p];
+  }
+  while (p < n) {
+    const long q = p + step;
+    double2 xn, vn[VC];
+    if (q < n) {
+      xn = wb[q];
+#pragma unroll
+      for (int c = 0; c < VC; ++c)
+        if (c < nv) vn[c] = Vb[c * vs + q];
+    }
+#pragma unroll
+    for (int c = 0; c < VC; ++c) {
+      if (c < nv) {
+        sum[2 * c] = fma(v[c].x, x.x, fma(v[c].y, x.y, sum[2 * c]));
+        sum[2 * c + 1] = fma(v[c].x, x.y, fma(-v[c].y, x.x, sum[2 * c + 1]));
+      }
+    }
+    p = q;
+    x = xn;
+#pragma unroll
+    for (int c = 0; c < VC; ++c) v[c] = vn[c];
+  }
+  __shared__ double sh[(KT / 32 + 1) * 2 * VC];
+  block_sum<2 * VC>(sum, sh);
+  if (threadIdx.x < nv) {
+    const double* s = sh + KT / 32 * 2 * VC + 2 * threadIdx.x;
+    partial[(long(b) * (j + 1) + i0 + threadIdx.x) * gridDim.x + blockIdx.x] =
+        make_double2(s[0], s[1]);
+  }
+}
+
+// w -= sum_{i <= j} sigma_i^2 S[b][i] V_i; with partial: |w|^2 sums, and the
+// new w as basis vector (unless Vnew is null).
+__global__ void __launch_bounds__(KT)
+update_kernel(const double2* __restrict__ V, long ldb, double2* __restrict__ w, long wstride,
+              long n, int j, const double2* __restrict__ S, int ldS, const double* __restrict__ sigma,
+              int ldsig, const int* __restrict__ active, double* __restrict__ partial,
+              double2* __restrict__ Vnew) {
+  pdl_wait();
+  const int b = blockIdx.y;
+  if (!active[b]) return;
+  __shared__ double2 coef[HZ_MAX_RESTART];
+  for (int i = threadIdx.x; i <= j; i += KT) {
+    const double s = sigma[long(i) * ldsig + b];
+    const double2 h = S[long(b) * ldS + i];
+    coef[i] = make_double2(s * s * h.x, s * s * h.y);
+  }
+  __syncthreads();
+  double nrm[1] = {0.0};
+  double2* wb = w + b * wstride;
+  const double2* Vb = V + long(b) * n;
+  const long vs = ldb * n;  // stride between basis vectors
+  for (long p = long(blockIdx.x) * KT + threadIdx.x; p < n; p += long(gridDim.x) * KT) {
+    // two interleaved partial sums
+    double dr0 = 0.0, di0 = 0.0, dr1 = 0.0, di1 = 0.0;
+    int i = 0;
+    for (; i + 3 <= j; i += 4) {
+      const double2 v0 = Vb[(i + 0) * vs + p], v1 = Vb[(i + 1) * vs + p];
+      const double2 v2 = Vb[(i + 2) * vs + p], v3 = Vb[(i + 3) * vs + p];
+      const double2 c0 = coef[i], c1 = coef[i + 1], c2 = coef[i + 2], c3 = coef[i + 3];
+      dr0 = fma(c0.x, v0.x, fma(-c0.y, v0.y, dr0));
+      di0 = fma(c0.x, v0.y, fma(c0.y, v0.x, di0));
+      dr1 = fma(c1.x, v1.x, fma(-c1.y, v1.y, dr1));
+      di1 = fma(c1.x, v1.y, fma(c1.y, v1.x, di1));
+      dr0 = fma(c2.x, v2.x, fma(-c2.y, v2.y, dr0));
+      di0 = fma(c2.x, v2.y, fma(c2.y, v2.x, di0));
+      dr1 = fma(c3.x, v3.x, fma(-c3.y, v3.y, dr1));
+      di1 = fma(c3.x, v3.y, fma(c3.y, v3.x, di1));
+    }
+    for (; i <= j; ++i) {
+      const double2 v = Vb[i * vs + p];
+      const double2 c = coef[i];
+      dr0 = fma(c.x, v.x, fma(-c.y, v.y, dr0));
+      di0 = fma(c.x, v.y, fma(c.y, v.x, di0));
+    }
+    double2 x = wb[p];
+    x.x -= dr0 + dr1;
+    x.y -= di0 + di1;
+    wb[p] = x;
+    if (Vnew) Vnew[long(b) * n + p] = x;
+    if (partial) nrm[0] = fma(x.x, x.x, fma(x.y, x.y, nrm[0]));
+  }
+  if (partial) {
+    __shared__ double sh[KT / 32 + 1];
+    block_sum<1>(nrm, sh);
+    if (threadIdx.x == 0) partial[long(b) * gridDim.x + blockIdx.x] = sh[KT / 32];
+  }
+}
+
+// out[b] = sum_{i < jn[b]} (sigma_i y_i) V_i
+__global__ void __launch_bounds__(KT)
+combine_kernel(const double2* __restrict__ V, long ldb, double2* __restrict__ out, long ostride,
+               long n, const double2* __restrict__ y, int ldy, const double* __restrict__ sigma,
+               int ldsig, const int* __restrict__ jn) {
+  pdl_wait();
+  const int b = blockIdx.y;
+  const int J = jn[b];
+  __shared__ double2 ys[HZ_MAX_RESTART];
+  for (int i = threadIdx.x; i < J; i += KT) {
+    const double s = sigma[long(i) * ldsig + b];
+    const double2 yy = y[long(b) * ldy + i];
+    ys[i] = make_double2(s * yy.x, s * yy.y);
+  }
+  __syncthreads();
+  double2* ob = out + b * ostride;
+  for (long p = long(blockIdx.x) * KT + threadIdx.x; p < n; p += long(gridDim.x) * KT) {
+    double2 x = make_double2(0.0, 0.0);
+    for (int i = 0; i < J; ++i) {
+      const double2 v = V[(long(i) * ldb + b) * n + p];
+      const double2 c = ys[i];
+      x.x = fma(c.x, v.x, fma(-c.y, v.y, x.x));
+      x.y = fma(c.x, v.y, fma(c.y, v.x, x.y));
+    }
+    ob[p] = x;
+  }
+}
+
 // w as basis vector: the first one of a cycle
+__global__ void __launch_bounds__(KT)
+copy_kernel(const double2* __restrict__ w, long wstride, long n, const int* __restrict__ active,
+            double2* __restrict__ V) {
+  pdl_wait();
+  const int b = blockIdx.y;
+  if (!active[b]) return;
+  for (long p = long(blockIdx.x) * KT + threadIdx.x; p < n; p += long(gridDim.x) * KT)
+    V[long(b) * n + p] = w[b * wstride + p];
+}
+
+// w as basis vector in block fixed point
 __global__ void __launch_bounds__(CT)
 encode_kernel(const double2* __restrict__ w, long wstride, long n, long ntiles,
               const int* __restrict__ active, int4* __restrict__ V, int* __restrict__ ev) {
@@ -809,13 +977,40 @@ hz_status launch_cgs(const Basis& Q, int nblk, int rows, double2* w, long wstrid
                      Vnew, enew));
   return HZ_OK;
 }
+
+// the FP64 basis
+double2* fp64(const Basis& Q, int i = 0) { return reinterpret_cast<double2*>(Q.V) + i * Q.ldb * Q.n; }
+
+hz_status launch_update_f64(const Basis& Q, double2* w, long wstride, int j, int nrhs,
+                            const double2* S, int ldS, const double* sigma, int ldsig,
+                            const int* active, double* partial, int* nblk, bool keep,
+                            cudaStream_t st) {
+  *nblk = krylov_blocks(Q.n, nrhs, 1);
+  HZ_CUDA(launch_pdl(update_kernel, dim3(*nblk, nrhs), dim3(KT), 0, st, fp64(Q), Q.ldb, w, wstride,
+                     Q.n, j, S, ldS, sigma, ldsig, active, partial,
+                     keep ? fp64(Q, j + 1) : static_cast<double2*>(nullptr)));
+  return HZ_OK;
+}
 }  // namespace
 
 hz_status launch_dots(const Basis& Q, double2* w, long wstride, int j, int nrhs, const int* active,
                       double2* partial, double2* S, int ldS, cudaStream_t st) {
-  const int nblk = cgs_blocks(Q.ntiles, nrhs, 4);
-  HZ_TRY(launch_cgs<CG_DOTS>(Q, nblk, CG_ROWS, w, wstride, j, nrhs, nullptr, 0, nullptr, 0, active, partial,
-                             nullptr, nullptr, st));
+  int nblk;
+  if (Q.fixed) {
+    nblk = cgs_blocks(Q.ntiles, nrhs, 4);
+    HZ_TRY(launch_cgs<CG_DOTS>(Q, nblk, CG_ROWS, w, wstride, j, nrhs, nullptr, 0, nullptr, 0, active,
+                               partial, nullptr, nullptr, st));
+  } else {
+    // balanced chunks of at most VC vectors, none empty; one wave of two blocks
+    // per SM, at least one point per thread
+    int nchunk = (j + VC) / VC;
+    const int vpc = (j + nchunk) / nchunk;
+    nchunk = (j + vpc) / vpc;
+    const long per = std::min(2 * 152 / (long(nrhs) * nchunk), (Q.n + KT - 1) / KT);
+    nblk = int(std::max(per, 1l));
+    HZ_CUDA(launch_pdl(dots_kernel, dim3(nblk, nrhs, nchunk), dim3(KT), 0, st, fp64(Q), Q.ldb, w,
+                       wstride, Q.n, j, vpc, active, partial));
+  }
   HZ_CUDA(launch_pdl(reduce_c_kernel, dim3(unsigned(nrhs * (j + 1))), dim3(KT), 0, st, partial,
                      nblk, j + 1, ldS, S));
   HZ_CUDA(cudaGetLastError());
@@ -826,6 +1021,13 @@ hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, in
                              const double2* S1, int ldS, const double* sigma, int ldsig,
                              const int* active, double2* partial, double2* S2,
                              cudaStream_t st) {
+  if (!Q.fixed) {
+    int unused;
+    HZ_TRY(launch_update_f64(Q, w, wstride, j, nrhs, S1, ldS, sigma, ldsig, active, nullptr, &unused,
+                             false, st));
+    count_launches(1);  // the phase counts two
+    return launch_dots(Q, w, wstride, j, nrhs, active, partial, S2, ldS, st);
+  }
   // One kernel while a tile's rows fit the shared memory of half an SM, with as
   // many blocks per SM as hold them: what it lacks is warps, not room for the
   // next tile's rows (2^24 points, j = 22: four blocks of 24 rows 1703 us, three
@@ -850,6 +1052,9 @@ hz_status launch_update_dots(const Basis& Q, double2* w, long wstride, int j, in
 hz_status launch_update(const Basis& Q, double2* w, long wstride, int j, int nrhs,
                         const double2* S, int ldS, const double* sigma, int ldsig,
                         const int* active, double* partial, int* nblk, bool keep, cudaStream_t st) {
+  if (!Q.fixed)
+    return launch_update_f64(Q, w, wstride, j, nrhs, S, ldS, sigma, ldsig, active, partial, nblk,
+                             keep, st);
   *nblk = cgs_blocks(Q.ntiles, nrhs, 4);
   HZ_TRY(launch_cgs<CG_UPDATE>(Q, *nblk, CG_ROWS, w, wstride, j, nrhs, S, ldS, sigma, ldsig, active,
                                reinterpret_cast<double2*>(partial),
@@ -861,8 +1066,12 @@ hz_status launch_update(const Basis& Q, double2* w, long wstride, int j, int nrh
 
 hz_status launch_encode(const Basis& Q, const double2* w, long wstride, int i, int nrhs,
                         const int* active, cudaStream_t st) {
-  HZ_CUDA(launch_pdl(encode_kernel, dim3(unsigned(Q.ntiles), nrhs), dim3(CT), 0, st, w, wstride,
-                     Q.n, Q.ntiles, active, Q.V + i * Q.ldb * Q.n, Q.ev + i * Q.ldb * Q.ntiles));
+  if (!Q.fixed)
+    HZ_CUDA(launch_pdl(copy_kernel, dim3(krylov_blocks(Q.n, nrhs, 1), nrhs), dim3(KT), 0, st, w,
+                       wstride, Q.n, active, fp64(Q, i)));
+  else
+    HZ_CUDA(launch_pdl(encode_kernel, dim3(unsigned(Q.ntiles), nrhs), dim3(CT), 0, st, w, wstride,
+                       Q.n, Q.ntiles, active, Q.V + i * Q.ldb * Q.n, Q.ev + i * Q.ldb * Q.ntiles));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
 }
@@ -890,8 +1099,12 @@ hz_status launch_solution_update(int zprec, const void* Z, long ldb, double2* u,
 
 hz_status launch_combine(const Basis& Q, double2* out, long ostride, int nrhs, const double2* y,
                          int ldy, const double* sigma, int ldsig, const int* jn, cudaStream_t st) {
-  HZ_TRY(launch_cgs<CG_COMBINE>(Q, cgs_blocks(Q.ntiles, nrhs, 4), CG_ROWS, out, ostride, 0, nrhs, y, ldy,
-                                sigma, ldsig, jn, nullptr, nullptr, nullptr, st));
+  if (Q.fixed)
+    HZ_TRY(launch_cgs<CG_COMBINE>(Q, cgs_blocks(Q.ntiles, nrhs, 4), CG_ROWS, out, ostride, 0, nrhs, y,
+                                  ldy, sigma, ldsig, jn, nullptr, nullptr, nullptr, st));
+  else
+    HZ_CUDA(launch_pdl(combine_kernel, dim3(krylov_blocks(Q.n, nrhs, 1), nrhs), dim3(KT), 0, st,
+                       fp64(Q), Q.ldb, out, ostride, Q.n, y, ldy, sigma, ldsig, jn));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
 }

@@ -146,7 +146,8 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
   const long ldb = B;
   KsDev& ks = p->ws->ks;
   // defined contents for the timed kernels: zero basis, unit scales, all active
-  const Basis Q{reinterpret_cast<int4*>(p->V), p->ev, ldb, n, (n + HZ_FX_TILE - 1) / HZ_FX_TILE};
+  const Basis Q{reinterpret_cast<int4*>(p->V), p->ev, ldb, n, (n + HZ_FX_TILE - 1) / HZ_FX_TILE,
+                p->opts.no_precond == 0};
   double2* W = p->V + long(m) * ldb * n;
   HZ_CUDA(cudaMemsetAsync(p->V, 0, size_t(j + 1) * B * n * sizeof(double2), st));
   HZ_CUDA(cudaMemsetAsync(W, 0, size_t(B) * n * sizeof(double2), st));
