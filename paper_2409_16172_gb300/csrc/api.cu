@@ -158,32 +158,41 @@ static hz_status ensure_planes(hz_plan* p, int prec) {
   return HZ_OK;
 }
 
-// Shape of the complex64 symbol pass for a last axis of N points and `points`
-// points over all right-hand sides, as (nodes per block, columns per thread).
-// Blocks of four nodes read the spectrum once for four planes and pay where
-// there are enough blocks without them (512^2 x 16 right-hand sides 266 -> 247 us, 2048^2 559 -> 509, 64^3 x 8 162 -> 149; but
-// 1024^2 104 -> 113); columns of 128 and 256 loop over more nodes with the
-// spectrum in shared memory (256^3 1390 -> 1178, 128^3 x 4 572 -> 554).  A pair of columns needs the registers
-// of two lines: threads with 24 or 30 elements (factors 3 and 5) do better
-// with one column on small grids (192^2 20.8 -> 17.6 us, 360 x 480 41 -> 34,
-// 720^2 122 -> 111) and with half blocks or four nodes on large ones
-// (192^3 734 -> 674, 180^3 988 -> 750, 240^3 2520 -> 1902), except at 960,
-// 1440 and 2880 (1440^2 336 -> 369).
-static void sym_shape(int N, long points, int* kpb, int* pair) {
+// Shape of the complex64 symbol pass for a last axis of N points, n points a
+// right-hand side and `points` over all of the plan's, as (nodes per block,
+// columns per thread).  By the plan's right-hand sides and not the call's, so
+// that a result does not depend on how many a call has.
+//   Four nodes a block read the spectrum once for four planes: worth it where
+//     there are blocks enough without them (512^2 x 16 right-hand sides
+//     266 -> 247 us, 2048^2 559 -> 509, 64^3 x 8 162 -> 149; but 1024^2
+//     104 -> 113).
+//   Columns of 128 and 256 loop over more nodes, the spectrum in shared memory
+//     (256^3 1390 -> 1178, 128^3 x 4 572 -> 554).
+//   Both only where one right-hand side alone has blocks enough too: a plan
+//     for 64 of 256^2 applied to one took 26 us in the looped form, 17 in the
+//     plain one; with 2^18 points (four nodes) or 2^20 (loop) a call with one
+//     is within 4%.
+//   A pair of columns needs the registers of two lines: threads with 24 or 30
+//     elements (factors 3 and 5) do better with one column on small grids
+//     (192^2 20.8 -> 17.6, 360 x 480 41 -> 34, 720^2 122 -> 111) and with half
+//     blocks or four nodes on large ones (192^3 734 -> 674, 180^3 988 -> 750,
+//     240^3 2520 -> 1902), except at 960, 1440 and 2880 (1440^2 336 -> 369).
+static void sym_shape(int N, long n, long points, int* kpb, int* pair) {
   *kpb = 1;
   *pair = 1;
+  const bool four = n >= (1l << 18);
   if (N % 5 == 0) {
     if (N <= 720 || N == 1920) {
       *pair = 0;
-      if (N <= 720 && points >= (1l << 22)) *kpb = 4;
-    } else if (N == 2400 && points >= (1l << 22)) {
+      if (four && N <= 720 && points >= (1l << 22)) *kpb = 4;
+    } else if (four && N == 2400 && points >= (1l << 22)) {
       *kpb = 4;
     }
   } else if (N == 96 || N == 192) {
     *pair = points < (1l << 17) ? 0 : 2;
-  } else if (N <= 256 && N >= 128 && points >= (1l << 22)) {
+  } else if (N <= 256 && N >= 128 && n >= (1l << 20) && points >= (1l << 22)) {
     *kpb = N == 256 ? 16 : 8;  // line_sym_inv_loop_kernel
-  } else if (points >= (1l << 21)) {
+  } else if (four && points >= (1l << 21)) {
     if (N == 256 || N == 512 || N == 2048) *kpb = 4;
     if (N == 64) {
       *kpb = 4;
@@ -210,7 +219,7 @@ hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* s
   const AxisTables& ty = m->ax[1];
   auto tw = [&](const AxisTables& t) -> const void* { return prec == 0 ? (const void*)t.tw64 : (const void*)t.tw32; };
   int kpb = 1, pair = 1;
-  if (by_size) sym_shape(m->dim == 2 ? ny : nz, n * p->max_nrhs, &kpb, &pair);
+  if (by_size) sym_shape(m->dim == 2 ? ny : nz, n, n * p->max_nrhs, &kpb, &pair);
   if (p->tune.syminv_kpb > 0) kpb = p->tune.syminv_kpb;
   if (p->tune.col_pair >= 0) pair = p->tune.col_pair;
   auto tw2 = [&](const AxisTables& t) -> const void* {
