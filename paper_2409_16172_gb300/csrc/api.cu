@@ -203,9 +203,10 @@ static void sym_shape(int N, long n, long points, int* kpb, int* pair) {
 
 // in: nrhs c128 vectors at stride n, each scaled by scale[b] (NULL = 1).
 // out_kind 0: c64 output, 1: c128 output.  prec 0: complex128 arithmetic.
-// by_size: untuned complex64 passes take their shape by size (applies); solves
-// keep one shape, because another rounding of the complex64 preconditioner
-// moves a solution by up to 1e-8 of its norm (1024^2, 100 Arnoldi steps).
+// by_size: complex64 passes of a plan whose shapes nobody chose take them by
+// size (applies); solves keep one shape, because the shapes differ in the last
+// bits and another rounding of the complex64 preconditioner moves a solution
+// by up to 1e-8 of its norm (1024^2, 100 Arnoldi steps).
 hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* scale, int nrhs,
                         void* out, int out_kind, cudaStream_t st, const int* active,
                         bool by_size) {
@@ -218,10 +219,9 @@ hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* s
   const AxisTables& tx = m->ax[0];
   const AxisTables& ty = m->ax[1];
   auto tw = [&](const AxisTables& t) -> const void* { return prec == 0 ? (const void*)t.tw64 : (const void*)t.tw32; };
-  int kpb = 1, pair = 1;
+  by_size = by_size && p->tune.by_size;
+  int kpb = p->tune.syminv_kpb, pair = p->tune.col_pair;
   if (by_size) sym_shape(m->dim == 2 ? ny : nz, n, n * p->max_nrhs, &kpb, &pair);
-  if (p->tune.syminv_kpb > 0) kpb = p->tune.syminv_kpb;
-  if (p->tune.col_pair >= 0) pair = p->tune.col_pair;
   auto tw2 = [&](const AxisTables& t) -> const void* {
     return prec == 1 && pair ? (const void*)t.tw32p : nullptr;
   };
@@ -243,7 +243,7 @@ hz_status precond_apply(hz_plan* p, int prec, const double2* in, const double* s
   // (1024^2 with K = 8: 67 -> 70).  By the plan's right-hand sides, so that a
   // result does not depend on how many a call has.
   int mode = p->tune.rowinv_mode;
-  if (mode == 0 && by_size && prec == 1 && !m->generic && rows * p->max_nrhs <= 4096 &&
+  if (by_size && prec == 1 && !m->generic && rows * p->max_nrhs <= 4096 &&
       !((nx == 512 || nx == 1024) && m->rowk_used < 7.0 * double(rows)))
     mode = 3;
   // the scattering x-inverse pass adds into out: cleared by the x-forward pass

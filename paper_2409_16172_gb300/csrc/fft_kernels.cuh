@@ -816,12 +816,13 @@ line_sym_inv_pair_kernel(const float2* __restrict__ vhat, float2* __restrict__ p
 
 // The paired symbol pass with a block's part of the spectrum in shared memory
 // (each thread's own elements, so without a barrier) and a loop over kpb
-// nodes: the same arithmetic as line_sym_inv_pair_kernel.  One-node blocks
-// wait on the spectrum's loads from L2 (long scoreboard 4.1 of 9.3 cycles per
-// issue at 256^3); blocks that keep it in registers over four nodes have half
-// the warps.  Whole apply at 256^3, K = 16: one node per block 1390 us, four
-// in registers 1250, this 1178; 128^3 x 4 right-hand sides 572, 583, 554;
-// 512-point columns no better than four in registers.
+// nodes: line_sym_inv_pair_kernel's formulas, but not its bits (planes differ
+// by up to 2e-7 of the largest value, as between one and four nodes a block).
+// One-node blocks wait on the spectrum's loads from L2 (long scoreboard 4.1 of
+// 9.3 cycles per issue at 256^3); blocks that keep it in registers over four
+// nodes have half the warps.  Whole apply at 256^3, K = 16: one node per block
+// 1390 us, four in registers 1250, this 1178; 128^3 x 4 right-hand sides 572,
+// 583, 554; 512-point columns no better than four in registers.
 template <int N, int TB, bool HERM>
 __global__ void __launch_bounds__(TB * LineCfg<float, N>::template tpl_p<1>(), 3)
 line_sym_inv_loop_kernel(const float2* __restrict__ vhat, float2* __restrict__ planes, int nx,

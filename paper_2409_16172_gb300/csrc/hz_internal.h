@@ -257,12 +257,15 @@ struct SolveWs;
 
 // Launch shapes the autotuner chooses per plan (defaults are the untuned
 // choice): nodes per block of the last-axis symbol pass, form of the
-// x-inverse, columns per thread.
+// x-inverse, columns per thread.  by_size: direct applies take theirs by size
+// instead (sym_shape); off once a caller has set shapes, or the autotuner has
+// found faster ones.
 struct Tune {
-  int syminv_kpb = 0;   // 0: by size (sym_shape)
+  int syminv_kpb = 1;
   int rowinv_mode = 0;  // FftOps::row_inv_acc mode (0..3)
-  int col_pair = -1;    // complex64 symbol pass: two columns per thread (2: in
-                        // half-size blocks); -1: by size
+  int col_pair = 1;     // complex64 symbol pass: two columns per thread (2: in
+                        // half-size blocks), 0: one
+  bool by_size = true;
 };
 }
 

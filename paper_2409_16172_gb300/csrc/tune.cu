@@ -114,6 +114,7 @@ extern "C" hz_status hz_plan_set_tune(hz_plan* plan, const hz_tune_report* r) {
   plan->tune.syminv_kpb = r->syminv_kpb;
   plan->tune.rowinv_mode = r->rowinv_mode;
   plan->tune.col_pair = r->col_pair;
+  plan->tune.by_size = false;
   return HZ_OK;
 }
 
@@ -179,9 +180,10 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
   float tbest = 1e30f;
   const int prec = p->opts.precision;
   void* out = p->Z;
-  p->tune = def;  // the untuned choice
+  best.by_size = false;
+  p->tune = def;  // what an untuned plan's apply does
   const float tdef = tm.best_ms([&] {
-    return precond_apply(p, prec, W, nullptr, B, out, prec == 1 ? 0 : 1, st, nullptr);
+    return precond_apply(p, prec, W, nullptr, B, out, prec == 1 ? 0 : 1, st, nullptr, true);
   });
   for (int pair : {1, 2, 0}) {
     if (pair != 1 && prec == 0) continue;  // FP64 has one form
@@ -216,7 +218,10 @@ extern "C" hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_repor
       best.rowinv_mode = mode;
     }
   }
-  r.apply_us = 1e3f * tbest;
+  // direct applies keep their shape by size where no candidate beats it (the
+  // node loop of sym_shape is not among them)
+  best.by_size = tdef <= tbest;
+  r.apply_us = 1e3f * std::min(tbest, tdef);
   r.apply_us_default = 1e3f * tdef;
   HZ_CUDA(cudaStreamSynchronize(st));
   p->tune = best;
