@@ -260,16 +260,6 @@ __device__ __forceinline__ long long int_of(double x, int E, int top) {
   const long long s = hi >> 31;
   return (static_cast<long long>((t + 1) >> 1) ^ s) - s;
 }
-// t 2^k: zero below the normal range, infinity above it
-__device__ __forceinline__ double double_of(long long t, int k) {
-  const double d = static_cast<double>(t);
-  const int hi = __double2hiint(d);
-  const int e = ((hi >> 20) & 0x7ff) + k;
-  double r = __hiloint2double(hi + (k << 20), __double2loint(d));
-  if (e >= 0x7ff) r = __hiloint2double((hi & 0x80000000) | 0x7ff00000, 0);
-  return (t == 0 || e <= 0) ? 0.0 : r;
-}
-
 // A block of LINES lines of N points.  ROWS: lines one after the other, else
 // interleaved (columns).
 template <int N_, int LINES_, bool ROWS> struct IBlock {

@@ -66,12 +66,29 @@ __device__ __forceinline__ long long fx_sum(long long hh, long long x) {
 // to E
 __device__ __forceinline__ int fx_unit(int E) { return E + 54 - 2 * FX_TOP - 2 * 1023; }
 
-// t 2^k; a result below the normal range is zero
+// t 2^k: zero below the normal range; above it (the operator's tiles keep
+// clear of it) a wrong value
 __device__ __forceinline__ double fx_to(long long t, int k) {
   const double d = static_cast<double>(t);
   const int hi = __double2hiint(d);
   const int e = ((hi >> 20) & 0x7ff) + k;
   return (t == 0 || e <= 0) ? 0.0 : __hiloint2double(hi + (k << 20), __double2loint(d));
 }
+// the same with infinity above the range
+__device__ __forceinline__ double double_of(long long t, int k) {
+  const double d = static_cast<double>(t);
+  const int hi = __double2hiint(d);
+  const int e = ((hi >> 20) & 0x7ff) + k;
+  double r = __hiloint2double(hi + (k << 20), __double2loint(d));
+  if (e >= 0x7ff) r = __hiloint2double((hi & 0x80000000) | 0x7ff00000, 0);
+  return (t == 0 || e <= 0) ? 0.0 : r;
+}
+
+// Infinities and NaN have no integer form: a tile that holds one has exponent
+// FX_INF, and sums over it are NaN.
+constexpr int FX_INF = 0x7ff;
+constexpr int FX_BAD = 1 << 14;  // above any sum of two exponents
+__device__ __forceinline__ int fx_exp_sum(int e, int f) { return max(e, f) >= FX_INF ? FX_BAD : e + f; }
+__device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
 
 }  // namespace hz

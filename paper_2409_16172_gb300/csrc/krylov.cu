@@ -311,7 +311,7 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
   };
   double2 xn = load_w(tile);
   if (UPD) {
-    warp_max(tid <= j ? ec + e0 : 0, redF);
+    warp_max(tid <= j ? fx_exp_sum(ec, e0) : 0, redF);
     __syncthreads();
     F = max_of(redF);
     if (tid <= j) cl[tid] = coef_limbs(ci, F - e0);
@@ -369,12 +369,13 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
       }
       a.join(a2);
       const int k = fx_unit(F);
-      const double dr = fx_to(a.re(), k), di = fx_to(a.im(), k);
+      double dr = double_of(a.re(), k), di = double_of(a.im(), k);
+      if (F >= FX_BAD) dr = di = fx_nan();
       x = MODE == CG_COMBINE ? make_double2(dr, di) : make_double2(x.x - dr, x.y - di);
       if (in) wb[p] = x;
       else x = make_double2(0.0, 0.0);
       if (MODE == CG_UPDATE) nrm[0] = fma(x.x, x.x, fma(x.y, x.y, nrm[0]));
-      warp_max(tid <= j ? ec + e1 : 0, redF);
+      warp_max(tid <= j ? fx_exp_sum(ec, e1) : 0, redF);
     }
     if (MODE != CG_COMBINE) warp_max(fx_exp(x), redw);
     __syncthreads();
@@ -426,8 +427,8 @@ cgs_kernel(const int4* __restrict__ V, const int* __restrict__ ev, long ldb, lon
         if ((lane & 3) == 0 && is <= j) {
           const int k = fx_unit(E + e);
           double2 s = sacc[is];
-          s.x += fx_to(sr, k);
-          s.y += fx_to(si, k);
+          s.x += max(E, e) < FX_INF ? double_of(sr, k) : fx_nan();
+          s.y += max(E, e) < FX_INF ? double_of(si, k) : fx_nan();
           sacc[is] = s;
         }
       }
