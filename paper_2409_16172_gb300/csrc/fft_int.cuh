@@ -31,6 +31,7 @@
 
 #include "fft_engine.cuh"
 #include "fixed.cuh"
+#include "recip.cuh"
 
 namespace hz {
 
@@ -488,15 +489,6 @@ iline_kernel(double2* data, int nx, int ntile, long S, long ostride, long bstrid
   int_transform<B, SIGN>(sm, red, E, tw, [&](int col, int p, double re, double im) {
     if (col < have) base[p * Si + col] = E < 0x7ff ? make_double2(re, im) : make_double2(nan, nan);
   });
-}
-
-// 1/x for the symbol: the MUFU approximation (about 20 bits) and one step of
-// third order, r (1 + e + e^2) with e = 1 - x r
-__device__ __forceinline__ double recip3(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
 }
 
 // Last axis: spectrum times q_k (Eqn. 021), inverse, plane k on the rows /

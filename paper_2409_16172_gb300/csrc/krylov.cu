@@ -26,6 +26,7 @@
 #include "fixed.cuh"
 #include "hz_internal.h"
 #include "kernels.h"
+#include "recip.cuh"
 
 namespace hz {
 namespace {
@@ -666,17 +667,6 @@ __device__ __forceinline__ double2 cmul_d(double2 a, double2 b) {
 __device__ __forceinline__ double2 cfma_d(double2 a, double2 b, double2 c) {  // a b + c
   return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
 }
-// 1/sqrt(x) for x > 0: the MUFU approximation (about 20 bits) and one step of
-// third order, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - x y^2.  Every FP64
-// instruction of a warp holds the sub-partition's FP64 unit for ~64 cycles;
-// this takes fewer of them than a square root followed by a division, or than
-// second-order steps.
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y, e * fma(0.375, e, 0.5), y);
-}
 // max(|a|, |b|) of finite doubles as an integer max of the magnitude bits
 // (IEEE order of non-negative doubles is that of their bit patterns), off the
 // FP64 pipe
@@ -719,7 +709,7 @@ givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
       double q = wsum[1];
       for (int i = 2; i < GT / 32; ++i) q += wsum[i];
       shn[0] = q;  // |w|^2 after orthogonalisation
-      shn[1] = q > 0.0 ? rsqrt_nr(q) : 0.0;
+      shn[1] = q > 0.0 ? rsqrt3(q) : 0.0;
     }
     __syncthreads();
     __syncthreads();
@@ -811,7 +801,7 @@ givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
       // rho = sqrt(|a|^2 + hn^2); c = |a| / rho; s = (a / |a|) hn / rho;
       // r = (a / |a|) rho
       const double rho2 = aa2 + hn2;
-      const double inv_aa = rsqrt_nr(aa2), inv_rho = rsqrt_nr(rho2);
+      const double inv_aa = rsqrt3(aa2), inv_rho = rsqrt3(rho2);
       const double aa = aa2 * inv_aa, rho = rho2 * inv_rho;
       c = aa * inv_rho;
       const double2 ph = make_double2(a.x * inv_aa, a.y * inv_aa);
@@ -828,7 +818,7 @@ givens_kernel(KsDev ks, int j, const double* __restrict__ partial, int nblk) {
     g[j + 1] = gn;  // -conj(s) g_j
     g[j] = make_double2(c * gj.x, c * gj.y);
     const double gn2 = fma(gn.x, gn.x, gn.y * gn.y);
-    const double est = gn2 > 0.0 ? gn2 * rsqrt_nr(gn2) : 0.0;
+    const double est = gn2 > 0.0 ? gn2 * rsqrt3(gn2) : 0.0;
     ks.est[b] = est;
     shn[2] = est;
     ks.jend[b] = j + 1;
