@@ -109,19 +109,37 @@ stencil_kernel(const InT* __restrict__ x, double2* __restrict__ y, const double2
 //
 // A block owns 30 x TY (x TZ) points; with the halo these are 32-point rows,
 // converted once each into shared memory.  All values of the tile share one
-// binary exponent E, the largest of them: v = x 2^(FS_TOP + 1023 - E),
-// |v| < 2^57, so a value within a factor 2^4 of the largest of its
-// neighbourhood keeps all its bits.  Neighbour sums are exact; g =
+// binary exponent E, the largest of them: v = x 2^(fs_top + 1023 - E) to the
+// nearest integer, below 2^(fs_top + 1).  Neighbour sums are exact; g =
 // gamma^2 / h_x^2 and omega^2 are integers below 2^60 of a unit for the whole
-// medium, and the products of 31-bit limbs are exact up to the last shift.  A
-// tile whose values leave the range of normal numbers, or are all zero, takes
-// the FP64 formula.  It is bound by the integer multiply-add pipe, which also
-// takes the 64-bit additions (62 lanes per clock and SM, about 130 a point in
-// 2D).  2400^2 damped, c128 input: 180 -> 82 us (3.9 TB/s); 192^3, c64 input:
-// 277 -> 115 us (2.5 TB/s).
+// medium, and the products of 31-bit limbs are exact up to the last shift.
+//
+// What the rounding of the values costs a point beside larger ones:
+//   complex128, and weighted sums  half a unit 2^-fs_top 2^E in each value,
+//     weighted with 2 diag in all, is 2 eps (eps = 2^-53) of the neighbour sum's
+//     terms as long as their weighted magnitudes add up to
+//     diag 2^(E + 52 - fs_top) at least, separately in the real and the
+//     imaginary parts.  A row of 30 points with one below that is done again by
+//     the FP64 formula.  Gaussian noise has one such row in thousands.
+//   complex64, equal spacings  values have 24 bits: nothing, if none but zeros
+//     is below 2^-24 of the tile's largest.  Neighbour sums are then exact, the
+//     products exact to 2^-27 of a value's unit, and the result is shifted by
+//     its own size before it is cut.  Other tiles are done whole by the FP64
+//     formula.
+// So every component keeps the FP64 formula's bound, some eps times the
+// magnitudes of its own terms, however steep the field is.  A warp whose first
+// row is done again leaves all its rows to the FP64 formula.  A tile whose values
+// leave the range of normal numbers, or are all zero, is done by it too.
+// It is bound by the integer multiply-add pipe, which also takes the 64-bit
+// additions (62 lanes per clock and SM, about 130 a point in 2D).  2400^2 damped,
+// c128 input: 180 -> 88 us (3.6 TB/s), of which the check takes 6; 192^3, c64
+// input: 277 -> 112 us (2.6 TB/s).  Fields that are steep all over (e^-r/8 at
+// 2400^2) take 215 us, most of it FP64.
 // ---------------------------------------------------------------------------
 constexpr int SW = 8;          // warps per block
-constexpr int FS_TOP = 56;
+// bit of the leading one of a value with exponent E: neighbour sums stay below
+// 2^61, which in the unweighted form of 3D is 12 values
+__host__ __device__ constexpr int fs_top(bool d3, bool unit) { return d3 && unit ? 56 : 57; }
 constexpr int FS_KEEP = 3;     // bits of the result kept below 2^62 units
 
 template <bool D3> struct FsTile {
@@ -135,43 +153,49 @@ template <bool D3> struct FsTile {
 struct FxStencil {
   int w2h, w2l;                 // omega^2 in units of q_w
   int kh[4], kl[4];             // x, y, z, diagonal weights (general spacing)
+  unsigned share[3];            // x, y, z weights over the diagonal's, times 2^32
   int k_out;                    // result = T 2^(E + k_out)
-  double qg;                    // unit of g
+  int uq;                       // unit of g: 2^uq
 };
 
-__device__ __forceinline__ int exp_bits(double2 z) {
-  return max((__double2hiint(z.x) >> 20) & 0x7ff, (__double2hiint(z.y) >> 20) & 0x7ff);
-}
-__device__ __forceinline__ int exp_bits(float2 z) {
-  const int e = max((__float_as_int(z.x) >> 23) & 0xff, (__float_as_int(z.y) >> 23) & 0xff);
+// magnitude of a value, in order of size, from its high word; zero only for
+// zeros (and doubles below 2^-1042)
+__device__ __forceinline__ int mag_bits(double v) { return __double2hiint(v) & 0x7fffffff; }
+__device__ __forceinline__ int mag_bits(float v) { return __float_as_int(v) & 0x7fffffff; }
+// biased FP64 exponent of such a magnitude
+template <typename T> __device__ __forceinline__ int mag_exp(int m) {
+  if constexpr (std::is_same<T, double2>::value) return m >> 20;
+  const int e = m >> 23;
   return e == 0 ? 0 : (e == 0xff ? 0x7ff : e + 896);
 }
 __device__ __forceinline__ long long shr(long long v, int n) {  // n > 63: zero
   asm("shr.u64 %0, %0, %1;" : "+l"(v) : "r"(n));
   return v;
 }
-// Truncated fixed-point value for the exponent E >= exponent of x.  Zeros and
-// subnormals need no test: with E at least FS_EMIN their shift is past the
-// last bit.
+// Fixed-point value, rounded to nearest, for the exponent E >= exponent of x.
+// Zeros and subnormals need no test: with E at least FS_EMIN their shift is
+// past the last bit.
 template <typename T> __device__ constexpr int FS_EMIN = 128;
 template <> __device__ constexpr int FS_EMIN<float2> = 896 + 60;
-__device__ __forceinline__ long long to_fs(double x, int E) {
+template <int TOP> __device__ __forceinline__ long long to_fs(double x, int E) {
   const int hi = __double2hiint(x);
   const unsigned lo = unsigned(__double2loint(x));
   const int ex = (hi >> 20) & 0x7ff;
   const unsigned mh = unsigned((hi & 0xfffff) | 0x100000);
-  const unsigned th = __funnelshift_l(lo, mh, 4), tl = lo << 4;
-  const long long t = shr(static_cast<long long>(static_cast<unsigned long long>(th) << 32 | tl), E - ex);
+  const unsigned th = __funnelshift_l(lo, mh, TOP - 51), tl = lo << (TOP - 51);
+  const long long t =
+      (shr(static_cast<long long>(static_cast<unsigned long long>(th) << 32 | tl), E - ex) + 1) >> 1;
   const long long sg = hi >> 31;
   return (t ^ sg) - sg;
 }
-__device__ __forceinline__ long long to_fs(float x, int E) {
+template <int TOP> __device__ __forceinline__ long long to_fs(float x, int E) {
   const int u = __float_as_int(x);
   const int ex = (u >> 23) & 0xff;
   const int sg = u >> 31;
-  const int m = ((u & 0x7fffff) | 0x800000) << 1;
+  const int m = ((u & 0x7fffff) | 0x800000) << (TOP - 54);
   // magnitude first: an arithmetic shift of a negative value would floor
-  const long long t = shr(static_cast<long long>(static_cast<unsigned long long>(unsigned(m)) << 32), E - 896 - ex);
+  const long long t =
+      (shr(static_cast<long long>(static_cast<unsigned long long>(unsigned(m)) << 32), E - 896 - ex) + 1) >> 1;
   const long long s = sg;
   return (t ^ s) - s;
 }
@@ -183,12 +207,33 @@ __device__ __forceinline__ int lim_l(long long v) { return int(unsigned(v) & 0x7
 struct __align__(16) CLong {
   long long x, y;
 };
+__device__ __forceinline__ int high(long long v) { return int(v >> 32); }
+__device__ __forceinline__ int size(long long v, long long w) { return abs(high(v)) + abs(high(w)); }
 __device__ __forceinline__ CLong operator+(const CLong& p, const CLong& q) {
   return CLong{p.x + q.x, p.y + q.y};
 }
 
+// zero for zeros
+__device__ __forceinline__ long long bits(double2 z) {
+  return (__double_as_longlong(z.x) | __double_as_longlong(z.y)) << 1;
+}
+
+// bits below 2^62 units to keep of hh 2^62 + m 2^31, |m| < 2^63: all that
+// leave the sum below 2^63
+__device__ __forceinline__ int keep_bits(long long hh) {
+  const int h = high(hh);
+  return min(__clz(h ^ (h >> 31)) - 2, 28);
+}
+
+// Blocks per SM that the registers have to allow: as many as spill next to
+// nothing (2400^2 damped: three 98 us, four 92, five 88).
+template <typename InT, bool D3, bool UNIT> constexpr int fx_blocks_per_sm() {
+  if (D3) return std::is_same<InT, double2>::value || !UNIT ? 3 : 4;
+  return UNIT ? 5 : 4;
+}
+
 template <typename InT, bool RESID, bool D3, bool UNIT>
-__global__ void __launch_bounds__(32 * SW)
+__global__ void __launch_bounds__(32 * SW, (fx_blocks_per_sm<InT, D3, UNIT>()))
 stencil_fx_kernel(const InT* __restrict__ x, double2* __restrict__ y, const double2* __restrict__ f,
                   const int4* __restrict__ gs, const double* __restrict__ a, double omega, double w2,
                   double rho_y, double rho_z, double diag, FxStencil k, int nx, int ny, int nz,
@@ -196,8 +241,11 @@ stencil_fx_kernel(const InT* __restrict__ x, double2* __restrict__ y, const doub
                   const int* __restrict__ active, double* __restrict__ partial) {
   pdl_wait();
   using T = FsTile<D3>;
+  constexpr int TOP = fs_top(D3, UNIT);
+  // whether points are checked for small terms, and not the tile for small values
+  constexpr bool CHECK = std::is_same<InT, double2>::value || !UNIT;
   extern __shared__ CLong tile[];  // [RZ][RY][32]
-  __shared__ int red[SW];
+  __shared__ int red[CHECK ? 2 : 3][SW];
   const int b = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);
   double nrm = 0.0;
@@ -234,78 +282,111 @@ stencil_fx_kernel(const InT* __restrict__ x, double2* __restrict__ y, const doub
       }
     };
     InT v[T::PER];
-    int E = 0;
+    int mx = 0, my = 0;  // largest magnitudes of the real and the imaginary parts
+    unsigned least = ~0u;  // smallest magnitude but zeros, less one
 #pragma unroll
     for (int i = 0; i < T::PER; ++i)
       if (warp + i * SW < T::ROWS) v[i] = xb[point(warp + i * SW)];
 #pragma unroll
     for (int i = 0; i < T::PER; ++i)
-      if (warp + i * SW < T::ROWS) E = max(E, exp_bits(v[i]));
+      if (warp + i * SW < T::ROWS) {
+        mx = max(mx, mag_bits(v[i].x));
+        my = max(my, mag_bits(v[i].y));
+        if (!CHECK) least = min(least, min(unsigned(mag_bits(v[i].x)) - 1u, unsigned(mag_bits(v[i].y)) - 1u));
+      }
     fetch(warp);
-    E = __reduce_max_sync(0xffffffffu, E);
-    if (lane == 0) red[warp] = E;
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    my = __reduce_max_sync(0xffffffffu, my);
+    if (!CHECK) least = __reduce_min_sync(0xffffffffu, least);
+    if (lane == 0) {
+      red[0][warp] = mx;
+      red[1][warp] = my;
+      if (!CHECK) red[2][warp] = int(least);
+    }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < SW; ++i) E = max(E, red[i]);
-    const bool fx = E >= FS_EMIN<InT> && E < 1920;
+    for (int i = 0; i < SW; ++i) {
+      mx = max(mx, red[0][i]);
+      my = max(my, red[1][i]);
+      if (!CHECK) least = min(least, unsigned(red[2][i]));
+    }
+    const int E = mag_exp<InT>(max(mx, my));
+    const bool fx = E >= FS_EMIN<InT> && E < 1920 &&
+                    (CHECK || int((least + 1u) >> 23) >= (max(mx, my) >> 23) - 24);
+    if (fx) {
 #pragma unroll
-    for (int i = 0; i < T::PER; ++i) {
-      if (warp + i * SW < T::ROWS) {
-        CLong s;
-        if (fx) {
-          s = CLong{to_fs(v[i].x, E), to_fs(v[i].y, E)};
-        } else {
-          const double2 d = ld2(&v[i], 0);
-          s = CLong{__double_as_longlong(d.x), __double_as_longlong(d.y)};
-        }
-        tile[(warp + i * SW) * 32 + lane] = s;
-      }
+      for (int i = 0; i < T::PER; ++i)
+        if (warp + i * SW < T::ROWS)
+          tile[(warp + i * SW) * 32 + lane] = CLong{to_fs<TOP>(v[i].x, E), to_fs<TOP>(v[i].y, E)};
     }
     __syncthreads();
     const int ke = E + k.k_out;
     double2* yb = y + b * out_stride;
     const double2* fb = RESID ? f + b * out_stride : nullptr;
-    auto rows = [&](auto fxc) {
-    constexpr bool FX = decltype(fxc)::value;
+    // rows that the FP64 formula does: bit i for the warp's i-th
+    unsigned again = fx ? 0u : ~0u;
+    // what the magnitudes of a component's terms (high words) have to add up
+    // to; a component that is zero in the whole tile is exact
+    constexpr int LOW = (UNIT ? (D3 ? 6 : 4) : 1) << (52 - 32);
+    const int low_x = mx ? LOW : 0, low_y = my ? LOW : 0;
+    if (fx) {
 #pragma unroll 4
-    for (int q = warp; q < T::TY * T::TZ; q += SW) {
-      const unsigned o = on;
-      const int4 G = Gn;
-      const double an = aa;
-      if (!sn) break;  // rows past the grid: so are the warp's later ones
-      if (q + SW < T::TY * T::TZ) fetch(q + SW);
-      const int qz = D3 ? q / T::TY : 0, qy = D3 ? q - qz * T::TY : q;
-      const CLong* c = tile + ((D3 ? qz + 1 : 0) * T::RY + qy + 1) * 32 + lane;
-      const CLong v0 = c[0];
-      double yr, yi;
-      if constexpr (FX) {
+      for (int q = warp; q < T::TY * T::TZ; q += SW) {
+        const unsigned o = on;
+        const int4 G = Gn;
+        const double an = aa;
+        if (!sn) break;  // rows past the grid: so are the warp's later ones
+        if (q + SW < T::TY * T::TZ) fetch(q + SW);
+        const int qz = D3 ? q / T::TY : 0, qy = D3 ? q - qz * T::TY : q;
+        const CLong* c = tile + ((D3 ? qz + 1 : 0) * T::RY + qy + 1) * 32 + lane;
+        const CLong v0 = c[0];
         CLong L;
-        if (UNIT) {
-          L = (c[-1] + c[1]) + (c[-32] + c[32]);
-          if (D3) L = L + (c[-32 * T::RY] + c[32 * T::RY]);
-          L.x -= (D3 ? 6 : 4) * v0.x;
-          L.y -= (D3 ? 6 : 4) * v0.y;
-        } else {
-          // weights in units of 2^ke (host), result in units of 2^(59 + ke)
-          // (the lowest products are below 2^62 each: four fit unsigned)
-          long long hx = 0, mx = 0, hy = 0, my = 0;
-          unsigned long long lx = 0, ly = 0;
-          auto term = [&](const CLong& s, int kh, int kl) {
-            const int xh = lim_h(s.x), xl = lim_l(s.x), yh = lim_h(s.y), yl = lim_l(s.y);
-            hx += mul_w(kh, xh);
-            mx += mul_w(kh, xl) + mul_w(kl, xh);
-            lx += (unsigned long long)mul_w(kl, xl);
-            hy += mul_w(kh, yh);
-            my += mul_w(kh, yl) + mul_w(kl, yh);
-            ly += (unsigned long long)mul_w(kl, yl);
-          };
-          term(c[-1] + c[1], k.kh[0], k.kl[0]);
-          term(c[-32] + c[32], k.kh[1], k.kl[1]);
-          if (D3) term(c[-32 * T::RY] + c[32 * T::RY], k.kh[2], k.kl[2]);
-          term(v0, k.kh[3], k.kl[3]);
-          mx += (long long)(lx >> 31);
-          my += (long long)(ly >> 31);
-          L = CLong{(hx << 3) + (mx >> 28), (hy << 3) + (my >> 28)};
+        bool small = false;  // a component of the sum has small terms
+        {
+          const CLong l = c[-1], r = c[1], d = c[-32], u = c[32];
+          const CLong n = D3 ? c[-32 * T::RY] : CLong{0, 0}, f = D3 ? c[32 * T::RY] : CLong{0, 0};
+          int sx, sy;
+          if (UNIT) {
+            L = (l + r) + (d + u);
+            if (D3) L = L + (n + f);
+            L.x -= (D3 ? 6 : 4) * v0.x;
+            L.y -= (D3 ? 6 : 4) * v0.y;
+            sx = size(l.x, r.x) + size(d.x, u.x) + (D3 ? 6 : 4) * abs(high(v0.x));
+            sy = size(l.y, r.y) + size(d.y, u.y) + (D3 ? 6 : 4) * abs(high(v0.y));
+            if (D3) {
+              sx += size(n.x, f.x);
+              sy += size(n.y, f.y);
+            }
+          } else {
+            // weights in units of 2^ke (host), result in units of 2^(59 + ke)
+            // (the lowest products are below 2^62 each: four fit unsigned)
+            long long hx = 0, mx = 0, hy = 0, my = 0;
+            unsigned long long lx = 0, ly = 0;
+            auto term = [&](const CLong& s, int kh, int kl) {
+              const int xh = lim_h(s.x), xl = lim_l(s.x), yh = lim_h(s.y), yl = lim_l(s.y);
+              hx += mul_w(kh, xh);
+              mx += mul_w(kh, xl) + mul_w(kl, xh);
+              lx += (unsigned long long)mul_w(kl, xl);
+              hy += mul_w(kh, yh);
+              my += mul_w(kh, yl) + mul_w(kl, yh);
+              ly += (unsigned long long)mul_w(kl, yl);
+            };
+            sx = abs(high(v0.x));
+            sy = abs(high(v0.y));
+            auto pair = [&](const CLong& p, const CLong& q, int i) {
+              term(p + q, k.kh[i], k.kl[i]);
+              sx += int(__umulhi(unsigned(size(p.x, q.x)), k.share[i]));
+              sy += int(__umulhi(unsigned(size(p.y, q.y)), k.share[i]));
+            };
+            pair(l, r, 0);
+            pair(d, u, 1);
+            if (D3) pair(n, f, 2);
+            term(v0, k.kh[3], k.kl[3]);
+            mx += (long long)(lx >> 31) + (1ll << 27);
+            my += (long long)(ly >> 31) + (1ll << 27);
+            L = CLong{(hx << 3) + (mx >> 28), (hy << 3) + (my >> 28)};
+          }
+          if (CHECK) small = sx < low_x || sy < low_y;
         }
         // g L + omega^2 v
         const int ah = lim_h(L.x), al = lim_l(L.x), bh = lim_h(L.y), bl = lim_l(L.y);
@@ -313,49 +394,93 @@ stencil_fx_kernel(const InT* __restrict__ x, double2* __restrict__ y, const doub
         const int nz_ = -G.z, nw = -G.w;
         const long long rh = mad_w(k.w2h, vxh, mad_w(nz_, bh, mul_w(G.x, ah)));
         const long long ih = mad_w(k.w2h, vyh, mad_w(G.z, ah, mul_w(G.x, bh)));
-        // rounded at the last bit kept: |g L + omega^2 v| < 2^121.2, 62.2 bits left
-        constexpr long long half = 1ll << (30 - FS_KEEP);
+        // CHECK: rounded at the last bit kept; |g L + omega^2 v| < 2^121.7, 62.7 bits left
+        constexpr long long half = CHECK ? 1ll << (30 - FS_KEEP) : 0;
         long long rm = (mad_w(nw, bl, mul_w(G.y, al)) >> 31) + (mad_w(k.w2l, vxl, half << 31) >> 31);
         long long im = (mad_w(G.w, al, mul_w(G.y, bl)) >> 31) + (mad_w(k.w2l, vyl, half << 31) >> 31);
         rm = mad_w(G.x, al, mad_w(G.y, ah, mad_w(nz_, bl, mad_w(nw, bh, mad_w(k.w2h, vxl, mad_w(k.w2l, vxh, rm))))));
         im = mad_w(G.x, bl, mad_w(G.y, bh, mad_w(G.z, al, mad_w(G.w, ah, mad_w(k.w2h, vyl, mad_w(k.w2l, vyh, im))))));
-        yr = fx_to((rh << FS_KEEP) + (rm >> (31 - FS_KEEP)), ke);
-        yi = fx_to((ih << FS_KEEP) + (im >> (31 - FS_KEEP)), ke);
-      } else {
-        auto d = [&](int i) {
-          return make_double2(__longlong_as_double(c[i].x), __longlong_as_double(c[i].y));
-        };
-        const double2 l = d(-1), rr = d(1), dn = d(-32), up = d(32), m = d(0);
-        double sr = fma(rho_y, dn.x + up.x, l.x + rr.x), si = fma(rho_y, dn.y + up.y, l.y + rr.y);
+        double yr, yi;
+        if (CHECK) {
+          yr = fx_to((rh << FS_KEEP) + (rm >> (31 - FS_KEEP)), ke);
+          yi = fx_to((ih << FS_KEEP) + (im >> (31 - FS_KEEP)), ke);
+        } else {
+          const int kr = keep_bits(rh), ki = keep_bits(ih);
+          yr = fx_to((rh << kr) + (rm >> (31 - kr)), ke + FS_KEEP - kr);
+          yi = fx_to((ih << ki) + (im >> (31 - ki)), ke + FS_KEEP - ki);
+        }
+        const bool redo = CHECK && __any_sync(0xffffffffu, out && small);
+        again |= unsigned(redo) << (q / SW);
+        if (redo && q == warp) {  // a steep field: the other rows would be too
+          again = ~0u;
+          break;
+        }
+        if (a) {
+          const double2 m = ld2(xb, o);
+          const double wa = omega * an;
+          yr = fma(-wa, m.y, yr);
+          yi = fma(wa, m.x, yi);
+        }
+        if (RESID) {
+          const double2 fv = fb[o];
+          yr = fv.x - yr;
+          yi = fv.y - yi;
+          if (out && !redo) nrm = fma(yr, yr, fma(yi, yi, nrm));
+        }
+        if (out && !redo) yb[o] = make_double2(yr, yi);
+      }
+    }
+#pragma unroll 1
+    for (int q = warp; again && q < T::TY * T::TZ; q += SW, again >>= 1) {
+      if (!(again & 1u)) continue;
+      const int qz = D3 ? q / T::TY : 0, qy = D3 ? q - qz * T::TY : q;
+      if (!(y0 + qy < ny && (!D3 || z0 + qz < nz))) break;
+      const int own = ((D3 ? qz + 1 : 0) * T::RY) + qy + 1;  // row of the tile
+      const unsigned o = point(own);
+      const double2 m = ld2(xb, o), dn = ld2(xb, point(own - 1)), up = ld2(xb, point(own + 1));
+      double2 zd = make_double2(0.0, 0.0), zu = zd;
+      if (D3) {
+        zd = ld2(xb, point(own - T::RY));
+        zu = ld2(xb, point(own + T::RY));
+      }
+      // a row of zeros with neighbours of zeros gives zeros
+      const long long any = bits(m) | bits(dn) | bits(up) | bits(zd) | bits(zu);
+      const bool zero = !__any_sync(0xffffffffu, any != 0);
+      double sr = 0.0, si = 0.0;
+      if (!zero) {
+        const double2 l = make_double2(__shfl_up_sync(0xffffffffu, m.x, 1), __shfl_up_sync(0xffffffffu, m.y, 1));
+        const double2 rr = make_double2(__shfl_down_sync(0xffffffffu, m.x, 1), __shfl_down_sync(0xffffffffu, m.y, 1));
+        sr = fma(rho_y, dn.x + up.x, l.x + rr.x);
+        si = fma(rho_y, dn.y + up.y, l.y + rr.y);
         if (D3) {
-          const double2 zd = d(-32 * T::RY), zu = d(32 * T::RY);
           sr = fma(rho_z, zd.x + zu.x, sr);
           si = fma(rho_z, zd.y + zu.y, si);
         }
         sr = fma(-diag, m.x, sr);
         si = fma(-diag, m.y, si);
-        const double gx = fma(double(G.x), 2147483648.0, double(G.y)) * k.qg;
-        const double gy = fma(double(G.z), 2147483648.0, double(G.w)) * k.qg;
+      }
+      if (!out) continue;
+      double yr = 0.0, yi = 0.0;
+      if (!zero) {
+        const int4 G = gs[o];
+        const double gx = fx_to((static_cast<long long>(G.x) << 31) + G.y, k.uq);
+        const double gy = fx_to((static_cast<long long>(G.z) << 31) + G.w, k.uq);
         yr = fma(gx, sr, fma(-gy, si, w2 * m.x));
         yi = fma(gx, si, fma(gy, sr, w2 * m.y));
-      }
-      if (a) {
-        const double2 m = ld2(xb, o);
-        const double wa = omega * an;
-        yr = fma(-wa, m.y, yr);
-        yi = fma(wa, m.x, yi);
+        if (a) {
+          const double wa = omega * a[o];
+          yr = fma(-wa, m.y, yr);
+          yi = fma(wa, m.x, yi);
+        }
       }
       if (RESID) {
         const double2 fv = fb[o];
         yr = fv.x - yr;
         yi = fv.y - yi;
-        if (out) nrm = fma(yr, yr, fma(yi, yi, nrm));
+        nrm = fma(yr, yr, fma(yi, yi, nrm));
       }
-      if (out) yb[o] = make_double2(yr, yi);
+      yb[o] = make_double2(yr, yi);
     }
-    };
-    if (fx) rows(std::true_type{});
-    else rows(std::false_type{});
   }
   if (RESID) {
     __shared__ double sh[SW];
@@ -411,10 +536,11 @@ bool fx_consts(const StencilConsts& c, int dim, int uq, FxStencil* k) {
     const double kap[4] = {1.0, c.rho_y, c.rho_z, -c.diag};
     for (int i = 0; i < 4; ++i)
       limbs31(std::llrint(std::ldexp(kap[i], -weight_unit(c))), &k->kh[i], &k->kl[i]);
+    for (int i = 0; i < 3; ++i) k->share[i] = unsigned(std::ldexp(kap[i] / c.diag, 32));
   }
-  k->qg = std::ldexp(1.0, uq);
+  k->uq = uq;
   // a 31 x 31 bit product's high part counts 2^62 units; the sums keep FS_KEEP more bits
-  k->k_out = 62 - FS_KEEP + uq + ul - FS_TOP - 1023;
+  k->k_out = 62 - FS_KEEP + uq + ul - fs_top(dim == 3, unit) - 1023;
   return true;
 }
 
@@ -487,6 +613,8 @@ hz_status stencil_prepare(hz_medium* m, double zeta_max, cudaStream_t st) {
   const int uq = std::max(std::ilogb(gmax), std::ilogb(c.w2)) + 1 - 60;
   FxStencil k{};
   if (std::ldexp(gmin, -uq) < 4503599627370496.0 || !fx_consts(c, m->dim, uq, &k)) return HZ_OK;
+  // omega^2 x is one more term, whose rounding the others have to cover
+  if (c.w2 > c.diag * gmin) return HZ_OK;
   gfix_kernel<<<unsigned((m->n + 255) / 256), 256, 0, st>>>(m->gamma2, m->n, std::ldexp(1.0, -uq));
   count_launches(1);
   HZ_CUDA(cudaGetLastError());
