@@ -105,16 +105,31 @@ typedef struct {
 } hz_interp;
 
 /* Solver options.
- *   precision  0: plain FP64 path (complex128 preconditioner, GMRES storing
- *                 no Z: u = u0 + Q(V y));
- *              1: complex64 preconditioner inside flexible GMRES; Arnoldi,
- *                 operator and residuals stay FP64.
+ *   precision  0: complex128 throughout (GMRES storing no Z:
+ *                 u = u0 + Q(V y));
+ *              1: complex64 preconditioner inside flexible GMRES; vectors,
+ *                 operator, residuals, scalar products and the small systems
+ *                 stay complex128.
+ *              Much of the complex128 arithmetic is done in 64-bit integers
+ *              that share an exponent, which are faster here than FP64.  What
+ *              a caller may rely on: the operator keeps the FP64 formula's
+ *              bound point by point (hz_apply_operator); the transforms are as
+ *              accurate as FP64 ones, that is to rounding errors of one size
+ *              all over the grid (hz_apply_preconditioner); the basis vectors
+ *              of a preconditioned solve are held to 2^-54 of the largest of
+ *              128 neighbouring points, below what the transforms leave, and
+ *              their scalar products and combinations are exact in that form
+ *              to 2^-55 of the largest product.  The unpreconditioned method,
+ *              whose vectors know no transform, keeps an FP64 basis.
  *   restart    m, the Krylov dimension per cycle (1..128).
  *   tol        stop when ||f - P_N u||_2 / ||f||_2 <= tol (true residual).
  *   maxit      cap on the total number of Arnoldi steps.
- *   graphs     1: capture each full Arnoldi cycle once as a CUDA graph and
- *              replay it (worth it for small grids, where launches cost as
- *              much as the kernels); 0: launch step by step.
+ *   graphs     1: after a plan's third full Arnoldi cycle capture the cycle
+ *              as a CUDA graph (per right-hand-side count) and replay it from
+ *              then on (worth it for small grids, where launches cost as much
+ *              as the kernels; the first cycles run step by step, so that a
+ *              plan of few cycles does not pay for the capture); 0: launch
+ *              step by step.  The results are the same bit for bit.
  *   no_precond 1: plain GMRES(m) on P_N u = f without the preconditioner,
  *              all in FP64 (the unpreconditioned baseline the paper compares
  *              against in Section 5); 0: preconditioned by Q_M.
@@ -215,11 +230,16 @@ hz_status hz_plan_create(hz_medium* med, const hz_solver_opts* opts, int max_nrh
 /* Autotuner (the paper has no counterpart; it tunes this implementation's
  * launch shapes).  Times candidate launch shapes of the kernels that dominate
  * a solve on the plan's own buffers with CUDA events on `stream`: nodes per
- * block and columns per thread of the last-axis symbol pass, and whether the x-inverse pass accumulates the weighted sum as it
- * goes, transforms the planes in place and gathers the sum afterwards, or
- * transforms each (row, node) line on its own and adds it into the output.
- * The CGS2 kernels have one shape: dots_bps, dots_vc and upd_bps are accepted
- * and reported but choose nothing.  The choice is stored in the plan and cached per (grid, K, max_nrhs, restart, precision) for the
+ * block and columns per thread of the last-axis symbol pass, and whether the
+ * x-inverse pass accumulates the weighted sum as it goes, transforms the planes
+ * in place and gathers the sum afterwards, or transforms each (row, node) line
+ * on its own and adds it into the output.  With precision 0 the passes have one
+ * form, and the choice changes nothing.  The CGS2 kernels have one shape:
+ * dots_bps, dots_vc and upd_bps are accepted and reported but choose nothing.
+ * Direct applies of an untuned plan take their shapes by size; those of a tuned
+ * one keep that where no candidate is faster.  apply_us_default is the time of
+ * an untuned plan's apply, apply_us the tuned plan's.  The choice is stored in
+ * the plan and cached per (grid, K, max_nrhs, restart, precision) for the
  * process; later plans with the same key reuse it without timing.
  * Synchronous; overwrites the plan's work arrays (call before solving). */
 typedef struct {
@@ -244,11 +264,11 @@ typedef struct {
 
 hz_status hz_plan_autotune(hz_plan* plan, void* stream, hz_tune_report* report);
 
-/* Sets the plan's launch shapes from a report (e.g. one saved from an
- * earlier hz_plan_autotune): dots_vc in {2, 4, 8}, dots_bps in 1..4, upd_bps
- * in 1..8, syminv_kpb in {1, 2, 4}, rowinv_mode in {0, 1, 2, 3}, col_pair in
- * {0, 1, 2}; the timing
- * fields are ignored.  HZ_ERR_INVALID_ARG for any other value. */
+/* Sets the plan's launch shapes, for solves and direct applies, from a report
+ * (e.g. one saved from an earlier hz_plan_autotune): dots_vc in {2, 4, 8},
+ * dots_bps in 1..4, upd_bps in 1..8, syminv_kpb in {1, 2, 4}, rowinv_mode in
+ * {0, 1, 2, 3}, col_pair in {0, 1, 2}; the timing fields are ignored.
+ * HZ_ERR_INVALID_ARG for any other value. */
 hz_status hz_plan_set_tune(hz_plan* plan, const hz_tune_report* report);
 
 /* Bytes of device memory the plan holds. */
@@ -259,19 +279,24 @@ hz_status hz_destroy_plan(hz_plan* plan);
 /* y = P_N x (Eqn. 001 discretised as in Section 5: the 5-point (2D) or
  * 7-point (3D) centred second difference, periodic, with gamma^2 of
  * Eqn. Complex_wave_speed in the layer) for nrhs vectors, x != y, device
- * pointers.  The arithmetic is FP64 in both precisions, as the Krylov method
- * needs it: precision 0 reads x as c128; precision 1 reads x as c64 (the
+ * pointers.  Precision 0 reads x as c128; precision 1 reads x as c64 (the
  * form in which flexible GMRES stores its preconditioned vectors, widened
- * exactly to FP64).  y is always c128.  Errors: HZ_ERR_INVALID_ARG for null
- * or aliasing pointers, nrhs outside 1..max_nrhs, precision not 0 / 1, or a
- * current device other than the medium's. */
+ * exactly).  y is always c128, with FP64 accuracy in both precisions: each
+ * component is within 16 times 2^-53 of the sum of the magnitudes of its own
+ * terms, however much larger values near it are (grids of 2^17 points and more
+ * form the sums in integers, and in FP64 where those would not do).  Errors:
+ * HZ_ERR_INVALID_ARG for null or aliasing pointers, nrhs outside 1..max_nrhs,
+ * precision not 0 / 1, or a current device other than the medium's. */
 hz_status hz_apply_operator(hz_plan* plan, const void* x, void* y, int nrhs, int precision,
                             void* stream);
 
 /* y = Q_M x for nrhs c128 device vectors (x may equal y).  precision 0
  * computes in complex128, 1 in complex64 (input rounded to c64, output
  * widened to c128).  Eqn. 103 / 403 with one forward FFT, K symbol
- * multiplies each followed by an inverse FFT, and the weighted sum. */
+ * multiplies each followed by an inverse FFT, and the weighted sum.  As with
+ * any FFT, rounding errors are of one size all over the grid, some 2^-53
+ * (2^-24) times the result's largest values.  A right-hand side's result does
+ * not depend on how many others the call has. */
 hz_status hz_apply_preconditioner(hz_plan* plan, const void* x, void* y, int nrhs,
                                   int precision, void* stream);
 
@@ -308,7 +333,7 @@ hz_status hz_apply_preconditioner_noalloc(const hz_medium* med, const void* x, v
  * right-hand sides with the restarted GMRES of Section 5 ("GMRES
  * implementation"; the paper preconditions from the left, this library from
  * the right, flexibly for precision 1, so that tol applies to the true
- * unpreconditioned residual): CGS2 Arnoldi in FP64, complex Givens
+ * unpreconditioned residual): CGS2 Arnoldi, complex Givens
  * rotations, true-residual check after each cycle whose estimate reached
  * tol.  f and u are c128 arrays of
  * nrhs * n elements in device OR host memory (host buffers are staged
@@ -456,7 +481,7 @@ unsigned long long hz_launch_count(void);
 
 /* Measures this GPU's FP64 FMA throughput (GFLOP/s, 2 flops per FMA) with a
  * kernel of independent FMA chains filling every SM for about 0.1 s; the
- * denominator for the FP64-bound Krylov kernels.  Synchronous. */
+ * denominator for the kernels that the FP64 pipe bounds.  Synchronous. */
 hz_status hz_measure_fp64_peak(double* gflops);
 
 #ifdef __cplusplus

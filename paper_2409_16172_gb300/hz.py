@@ -287,9 +287,9 @@ class Plan:
         return {f: getattr(r, f) for f, _ in r._fields_}
 
     def set_tune(self, **shape) -> None:
-        """Set launch shapes (hz_plan_set_tune); unspecified ones keep the
-        defaults dots_vc=8, dots_bps=2, upd_bps=4, syminv_kpb=1, rowinv_mode=0,
-        col_pair=1."""
+        """Set launch shapes for solves and direct applies (hz_plan_set_tune);
+        unspecified ones are syminv_kpb=1, rowinv_mode=0, col_pair=1.  dots_vc,
+        dots_bps and upd_bps are accepted and choose nothing."""
         r = hz_tune_report()
         r.dots_vc, r.dots_bps, r.upd_bps, r.syminv_kpb, r.rowinv_mode = 8, 2, 4, 1, 0
         r.col_pair = 1
