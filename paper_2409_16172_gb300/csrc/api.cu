@@ -362,7 +362,7 @@ extern "C" hz_status hz_plan_create(hz_medium* med, const hz_solver_opts* opts, 
   // one budget for the tile exponents of the basis and the block partial
   // sums: the stencil residual (one double per block), the CGS2 dot partials
   // (2 (j+1) doubles per block) and the norms (one double per block)
-  const int nblk = std::max(int((n + 255) / 256), krylov_blocks(n, 1, 1));
+  const int nblk = std::max(int((n + 255) / 256), krylov_blocks(n, 1));
   const size_t budget = size_t(B) * (m + 2) * std::max(nblk, 1024) * 2;
   const size_t evlen = size_t(B) * m * ((n + HZ_FX_TILE - 1) / HZ_FX_TILE);
   p->partial_len = std::max(budget - (evlen + 1) / 2,

@@ -443,7 +443,7 @@ __device__ __forceinline__ void add_out(double2* p, double x, double y) {
 // between runs by rounding (the gather form does not).
 template <typename R, int N, typename OutT, int LPB, bool GEN>
 __global__ void __launch_bounds__(LPB * LineCfg<R, N>::TPL_ROW,
-                                  sizeof(R) == 4 && LPB * LineCfg<R, N>::TPL_ROW < 512
+                                  LPB * LineCfg<R, N>::TPL_ROW < 512
                                       ? 512 / (LPB * LineCfg<R, N>::TPL_ROW) : 1)
 row_inv_scatter_kernel(const typename cvec<R>::T* __restrict__ planes,
                        const typename RecT<R>::T* __restrict__ rec,

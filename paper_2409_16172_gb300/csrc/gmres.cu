@@ -157,7 +157,7 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
   if (!u_dev) HZ_CUDA(cudaMemcpyAsync(p->u, u_io, vbytes, cudaMemcpyHostToDevice, st));
 
   const int nblk_r = stencil_blocks(med);
-  const int nblk_n = krylov_blocks(n, nrhs, 1);
+  const int nblk_n = krylov_blocks(n, nrhs);
   const double Bn = double(nrhs) * n;
   {
     PhaseScope ps(st, PH_NORM, 16.0 * Bn, 4.0 * Bn, 2);
@@ -219,7 +219,7 @@ hz_status gmres_solve(hz_plan* plan, const void* f_in, void* u_io, int nrhs, hz_
     ctl.status = status.data();
     ctl.rel = rel.data();
     ctl.est = est.data();
-    const int nblk1 = krylov_blocks(n, 1, 1);
+    const int nblk1 = krylov_blocks(n, 1);
     ctl.admit = [&, nblk1](int b) -> hz_status {
       double nb = 0.0;
       HZ_TRY(launch_norm2(f + long(b) * n, n, n, 1, p->partial, nblk1, ks.bnorm + b, st));

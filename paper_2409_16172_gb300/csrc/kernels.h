@@ -90,7 +90,7 @@ hz_status launch_residual(const hz_medium* m, const double2* u, const double2* f
                           long stride, int nrhs, const int* active, double* partial,
                           cudaStream_t st);
 
-int krylov_blocks(long n, int nrhs, int nchunk);
+int krylov_blocks(long n, int nrhs);
 // Arnoldi basis: vector i of right-hand side b at V + (i ldb + b) n.  fixed:
 // in block fixed-point form (fixed.cuh), with tile exponents at
 // ev + (i ldb + b) ntiles; else in FP64.

@@ -921,20 +921,15 @@ norm2_kernel(const double2* __restrict__ x, long stride, long n, double* __restr
 
 }  // namespace
 
-// Blocks per right-hand side of the element-wise FP64 kernels: bps blocks
-// per SM over the whole launch, but at least one point per thread.  Short
-// vectors thus still spread over every SM: an FP64 warp instruction holds a
-// sub-partition's FP64 unit for ~64 cycles, so a few long-running warps
-// would serialise the work.
-int krylov_blocks_bps(long n, int nrhs, int nchunk, int bps) {
-  long per = (long(bps) * 152 + long(nrhs) * nchunk - 1) / (long(nrhs) * nchunk);
-  long maxb = (n + KT - 1) / KT;
-  if (per > maxb) per = maxb;
-  if (per < 1) per = 1;
-  return int(per);
+// Blocks per right-hand side of the element-wise FP64 kernels: four per SM over
+// the whole launch, but at least one point per thread.  Short vectors thus
+// still spread over every SM: an FP64 warp instruction holds a sub-partition's
+// FP64 unit for ~64 cycles, so a few long-running warps would serialise the
+// work.
+int krylov_blocks(long n, int nrhs) {
+  const long per = (4 * 152 + long(nrhs) - 1) / nrhs;
+  return int(std::max(std::min(per, (n + KT - 1) / KT), 1l));
 }
-
-int krylov_blocks(long n, int nrhs, int nchunk) { return krylov_blocks_bps(n, nrhs, nchunk, 4); }
 
 namespace {
 // Blocks per right-hand side of the Gram-Schmidt kernels: they walk over the
@@ -976,7 +971,7 @@ hz_status launch_update_f64(const Basis& Q, double2* w, long wstride, int j, int
                             const double2* S, int ldS, const double* sigma, int ldsig,
                             const int* active, double* partial, int* nblk, bool keep,
                             cudaStream_t st) {
-  *nblk = krylov_blocks(Q.n, nrhs, 1);
+  *nblk = krylov_blocks(Q.n, nrhs);
   HZ_CUDA(launch_pdl(update_kernel, dim3(*nblk, nrhs), dim3(KT), 0, st, fp64(Q), Q.ldb, w, wstride,
                      Q.n, j, S, ldS, sigma, ldsig, active, partial,
                      keep ? fp64(Q, j + 1) : static_cast<double2*>(nullptr)));
@@ -1058,7 +1053,7 @@ hz_status launch_update(const Basis& Q, double2* w, long wstride, int j, int nrh
 hz_status launch_encode(const Basis& Q, const double2* w, long wstride, int i, int nrhs,
                         const int* active, cudaStream_t st) {
   if (!Q.fixed)
-    HZ_CUDA(launch_pdl(copy_kernel, dim3(krylov_blocks(Q.n, nrhs, 1), nrhs), dim3(KT), 0, st, w,
+    HZ_CUDA(launch_pdl(copy_kernel, dim3(krylov_blocks(Q.n, nrhs), nrhs), dim3(KT), 0, st, w,
                        wstride, Q.n, active, fp64(Q, i)));
   else
     HZ_CUDA(launch_pdl(encode_kernel, dim3(unsigned(Q.ntiles), nrhs), dim3(CT), 0, st, w, wstride,
@@ -1077,7 +1072,7 @@ hz_status launch_givens(const KsDev& ks, int j, int nrhs, const double* partial,
 hz_status launch_solution_update(int zprec, const void* Z, long ldb, double2* u, long ustride,
                                  long n, int nrhs, const double2* y, int ldy, const int* jn,
                                  cudaStream_t st) {
-  const int nblk = krylov_blocks(n, nrhs, 1);
+  const int nblk = krylov_blocks(n, nrhs);
   if (zprec == 0)
     HZ_CUDA(launch_pdl(solution_update_kernel<double2>, dim3(nblk, nrhs), dim3(KT), 0, st,
                        static_cast<const double2*>(Z), ldb, u, ustride, n, y, ldy, jn));
@@ -1094,7 +1089,7 @@ hz_status launch_combine(const Basis& Q, double2* out, long ostride, int nrhs, c
     HZ_TRY(launch_cgs<CG_COMBINE>(Q, cgs_blocks(Q.ntiles, nrhs, 4), CG_ROWS, out, ostride, 0, nrhs, y,
                                   ldy, sigma, ldsig, jn, nullptr, nullptr, nullptr, st));
   else
-    HZ_CUDA(launch_pdl(combine_kernel, dim3(krylov_blocks(Q.n, nrhs, 1), nrhs), dim3(KT), 0, st,
+    HZ_CUDA(launch_pdl(combine_kernel, dim3(krylov_blocks(Q.n, nrhs), nrhs), dim3(KT), 0, st,
                        fp64(Q), Q.ldb, out, ostride, Q.n, y, ldy, sigma, ldsig, jn));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
@@ -1102,7 +1097,7 @@ hz_status launch_combine(const Basis& Q, double2* out, long ostride, int nrhs, c
 
 hz_status launch_scale_copy(const double2* V, const double* sigma, double2* out, long n, int nrhs,
                            const int* active, cudaStream_t st) {
-  const int nblk = krylov_blocks(n, nrhs, 1);
+  const int nblk = krylov_blocks(n, nrhs);
   HZ_CUDA(launch_pdl(scale_copy_kernel, dim3(nblk, nrhs), dim3(KT), 0, st, V, sigma, out, n,
                      active));
   HZ_CUDA(cudaGetLastError());
@@ -1111,7 +1106,7 @@ hz_status launch_scale_copy(const double2* V, const double* sigma, double2* out,
 
 hz_status launch_axpy(double2* u, const double2* t, long stride, long n, int nrhs, const int* jn,
                       cudaStream_t st) {
-  const int nblk = krylov_blocks(n, nrhs, 1);
+  const int nblk = krylov_blocks(n, nrhs);
   HZ_CUDA(launch_pdl(axpy_kernel, dim3(nblk, nrhs), dim3(KT), 0, st, u, t, stride, n, jn));
   HZ_CUDA(cudaGetLastError());
   return HZ_OK;
