@@ -115,10 +115,14 @@ extern "C" size_t hz_request_footprint(const hz_grid* g, const hz_interp* it,
   const size_t rows = size_t(n / g->n[0]);
   size_t med = size_t(n) * (16 + 8 + 4 + (has_a ? 8 : 0) + 16 + (generic ? 52 : 0)) +
                (rows + 1) * 16 * (generic ? 4 : 1) + rows * size_t(K) * 8 + (1 << 20);
+  // Z: the preconditioned vectors, at least one c128 vector where it is the
+  // work vector of an FP64, unpreconditioned or left step
+  const size_t z = o->precision == 1 ? size_t(m) * B * n * 8 : 0;
+  const bool work = o->precision == 0 || o->no_precond || o->left;
   size_t plan = B * n * 16                      // tmp
                 + B * K * n * es                // planes
                 + size_t(m + 1) * B * n * 16    // V
-                + (o->precision == 1 ? size_t(m) * B * n * 8 : B * n * 16)  // Z
+                + std::max(z, work ? B * n * 16 : 0)  // Z
                 + 2 * B * n * 16                // staged u, f
                 + fft_partial_bytes(n, int(B), m) + (1 << 20);
   return med + plan;
