@@ -132,7 +132,7 @@ stencil_kernel(const InT* __restrict__ x, double2* __restrict__ y, const double2
 // leave the range of normal numbers, or are all zero, is done by it too.
 // It is bound by the integer multiply-add pipe, which also takes the 64-bit
 // additions (62 lanes per clock and SM, about 130 a point in 2D).  2400^2 damped,
-// c128 input: 180 -> 88 us (3.6 TB/s), of which the check takes 6; 192^3, c64
+// c128 input: 180 -> 87 us (3.7 TB/s), of which the check takes 3; 192^3, c64
 // input: 277 -> 112 us (2.6 TB/s).  Fields that are steep all over (e^-r/8 at
 // 2400^2) take 215 us, most of it FP64.
 // ---------------------------------------------------------------------------
@@ -153,7 +153,7 @@ template <bool D3> struct FsTile {
 struct FxStencil {
   int w2h, w2l;                 // omega^2 in units of q_w
   int kh[4], kl[4];             // x, y, z, diagonal weights (general spacing)
-  unsigned share[3];            // x, y, z weights over the diagonal's, times 2^32
+  int share[3];                 // x, y, z weights over the diagonal's are 2^-share at least
   int k_out;                    // result = T 2^(E + k_out)
   int uq;                       // unit of g: 2^uq
 };
@@ -375,8 +375,8 @@ stencil_fx_kernel(const InT* __restrict__ x, double2* __restrict__ y, const doub
             sy = abs(high(v0.y));
             auto pair = [&](const CLong& p, const CLong& q, int i) {
               term(p + q, k.kh[i], k.kl[i]);
-              sx += int(__umulhi(unsigned(size(p.x, q.x)), k.share[i]));
-              sy += int(__umulhi(unsigned(size(p.y, q.y)), k.share[i]));
+              sx += size(p.x, q.x) >> k.share[i];
+              sy += size(p.y, q.y) >> k.share[i];
             };
             pair(l, r, 0);
             pair(d, u, 1);
@@ -536,7 +536,7 @@ bool fx_consts(const StencilConsts& c, int dim, int uq, FxStencil* k) {
     const double kap[4] = {1.0, c.rho_y, c.rho_z, -c.diag};
     for (int i = 0; i < 4; ++i)
       limbs31(std::llrint(std::ldexp(kap[i], -weight_unit(c))), &k->kh[i], &k->kl[i]);
-    for (int i = 0; i < 3; ++i) k->share[i] = unsigned(std::ldexp(kap[i] / c.diag, 32));
+    for (int i = 0; i < dim; ++i) k->share[i] = std::min(31, -std::ilogb(kap[i] / c.diag));
   }
   k->uq = uq;
   // a 31 x 31 bit product's high part counts 2^62 units; the sums keep FS_KEEP more bits
