@@ -57,6 +57,9 @@ ALPHA = 0.1
 # the GB300 by this benchmark's GPU arm; the reference arm cannot run the GPU
 # and scales its per-step time by these counts)
 GPU_STEPS_PER_SOLVE = {"cfg3": 95, "cfg2": 100, "cfg1": 29, "cfg4": 67}
+# DRAM traffic over algorithmic bytes of the dots and the fused update and dots
+# of one Arnoldi step (ncu, 128^3, 21 basis vectors: 1511.6 MB against 1510.0)
+DOTS_TRAFFIC_RATIO = 1.001
 
 
 def workload_config(p, name=DEFAULT_WORKLOAD, nrhs=1, symbol_kind=0):
@@ -432,7 +435,10 @@ def run_gpu(args, p, name):
     fp64_phases = {"cgs2_dots", "cgs2_update", "stencil", "residual", "solution_update", "norm"}
     achieved = d["bytes"] / d["ms"] / 1e6  # GB/s
     roof = {"kernel": kname, "bound": "hbm", "achieved": achieved, "peak": hbm,
-            "unit": "GB/s", "frac": achieved / hbm, "traffic": None,
+            "unit": "GB/s", "frac": achieved / hbm,
+            "traffic": DOTS_TRAFFIC_RATIO * d["bytes"] / d["launches"] if kname == "cgs2_dots" else None,
+            "traffic_note": "bytes per launch: DRAM read + write over algorithmic bytes of one ncu-captured "
+                            "step (128^3, 21 vectors), times the algorithmic bytes here",
             "peak_source": hbm_src, "launches": d["launches"],
             "avg_launch_us": 1e3 * d["ms"] / d["launches"],
             "timing": "CUDA events per launch, profiled pass of the same steps"}
